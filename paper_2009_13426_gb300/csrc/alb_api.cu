@@ -209,6 +209,8 @@ int alb_create(const alb_config* cfg, alb_handle** out) {
   p.half_gm1 = 0.5 * (cfg->gamma - 1.0);
   p.shakhov = cfg->prandtl != 1.0 ? 1 : 0;
   p.prandtl = cfg->prandtl;
+  p.icp = 1.0 / p.cp;
+  p.kappa_nu = cfg->nu / cfg->prandtl;
   for (int j = 0; j < 3; ++j) {
     p.seps[j] = cfg->sensor_eps[j];
     p.salpha[j] = cfg->sensor_alpha[j];

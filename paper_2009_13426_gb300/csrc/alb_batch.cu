@@ -177,10 +177,12 @@ cudaError_t GroupPlan::flip(cudaStream_t s) const { return launch_flip(d_cur_, n
     if (e_ != cudaSuccess) return cuda_error(e_, what);     \
   } while (0)
 
-// Default launch shape of a precision: variant 0, tiles no wider than it.
+// Default launch shape of a precision: the single-flow kernel's block in the FP32
+// form (variant 2, 256 x 2), variant 0 in FP64 plain; tiles 32 nodes wide.
 Tuning default_tuning(int precision) {
   Tuning t;
-  const int block = batch_variant(precision, 0).block;
+  if (precision == ALB_FP32_FORM) t.variant = 2;
+  const int block = batch_variant(precision, t.variant).block;
   for (int c = 0; c < 3; ++c) t.tile_w[c] = std::min(t.tile_w[c], block);
   return t;
 }
@@ -244,12 +246,12 @@ int tune_group(GroupPlan* p, cudaStream_t stream, int* counter, int trials) {
   for (FlowDev* f : p->flows()) present[size_class(f->prm.nx)] = true;
   Tuning best = p->tuning();
   float best_ms = 0.0f;
-  // 1. kernel variant, tiles as wide as the block
+  // 1. kernel variant, tiles 32 nodes wide
   for (int v = 0; v < batch_variant_count(prec) && rc == ALB_OK; ++v) {
     Tuning t = best;
     t.variant = v;
     const int block = batch_variant(prec, v).block;
-    for (int c = 0; c < 3; ++c) t.tile_w[c] = std::min(128, block);
+    for (int c = 0; c < 3; ++c) t.tile_w[c] = std::min(32, block);
     float ms = 0.0f;
     rc = try_tuning(stream, p, t, -1, trials, saved, counter, &ms);
     if (rc == ALB_OK && (v == 0 || ms < best_ms)) {

@@ -26,9 +26,8 @@ __global__ void __launch_bounds__(B, MINB)
   __shared__ __align__(16) unsigned long long s_args[sizeof(StepArgs<P>) / 8];
   __shared__ int s_item;
   __shared__ RebuildQueue<B> s_rq;
-  load_exptab(s_tab);  // includes a barrier
   const StepArgs<P>& a = *reinterpret_cast<const StepArgs<P>*>(s_args);
-  const Columns<P, B> cl(smem_raw);
+  const Columns<P, B> cl(smem_raw, s_tab);  // includes a barrier
   int it = blockIdx.x;
   int loaded = -1;  // (flow, buffer) whose arguments s_args holds
   for (;;) {
@@ -54,7 +53,7 @@ __global__ void __launch_bounds__(B, MINB)
       loaded = want;
     }
     NodeCount nc;
-    tile_step<P, B>(a, w.x0, w.y0, w.tw_log2, cl, s_tab, s_rq, nc);
+    tile_step<P, B>(a, w.x0, w.y0, w.tw_log2, cl, s_rq, nc);
     flush_counts(a.ctr, nc);
     if (!counter) it += gridDim.x;
   }

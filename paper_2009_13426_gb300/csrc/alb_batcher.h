@@ -12,7 +12,7 @@ namespace alb {
 // Launch shape of one precision (the C ABI's alb_batch_tuning).
 struct Tuning {
   int variant = 0;
-  int tile_w[3] = {64, 128, 128};  // flows with nx < 128, nx < 512, larger
+  int tile_w[3] = {32, 32, 32};  // flows with nx < 128, nx < 512, larger (see step_grid)
   int dynamic = 1;
   int blocks_per_sm = 0;           // 0: occupancy maximum
 };

@@ -70,6 +70,7 @@ struct Params {
   double overlap;    // widening of the current shift's range (0: Eq. criterion)
   double cv, cp;     // Cv = 1/(gamma-1), Cp = gamma Cv
   double half_gm1;   // (gamma - 1) / 2 = 1 / (2 Cv)
+  double icp, kappa_nu;  // 1 / Cp, nu / Pr (heat conduction: kappa = rho Cp nu / Pr)
   double seps[3], salpha[3];
   double skx[4], sky[4];  // sensor knots: log10(eps) and alpha (host-computed)
   double thr[6];          // criterion thresholds (t + 1) - n0, t = -umax .. umax - 1
@@ -143,6 +144,14 @@ __device__ __forceinline__ int select_shift_neighbours(double u, int axis, const
   return best;
 }
 
+// Product rounded by itself. The compiler may fuse a product and a sum into one
+// FMA or not, depending on the code around them; in the code that several
+// kernels share (single-flow and batched variants) every FMA is therefore
+// written out and every other product is one of these, so that a node's update
+// gives the same bits in all of them.
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // s + c * v with c a compile-time integer after unrolling: the zero and unit
 // cases fold away, keeping IEEE semantics for the rest.
 template <typename R>
@@ -175,22 +184,22 @@ __device__ __forceinline__ P sensor_alpha(const Params& pr, P eps) {
 #pragma unroll
   for (int k = 0; k < 3; ++k)
     if (l <= (P)pr.skx[k + 1])
-      return (P)pr.sky[k] + ((P)pr.sky[k + 1] - (P)pr.sky[k]) * (l - (P)pr.skx[k]) /
+      return (P)pr.sky[k] + mul_rn((P)pr.sky[k + 1] - (P)pr.sky[k], l - (P)pr.skx[k]) /
                                 ((P)pr.skx[k + 1] - (P)pr.skx[k]);
   return (P)pr.sky[3];
 }
 
 // Targets of Eqs. G0_8mom..G3yaa_8mom per unit density, lattice frame.
 __device__ __forceinline__ void targets(double ubx, double uby, double T, double m[NM]) {
-  const double u2 = ubx * ubx + uby * uby;
+  const double u2 = fma(ubx, ubx, mul_rn(uby, uby)), q = fma(4.0, T, u2);
   m[0] = 1.0;
   m[1] = ubx;
   m[2] = uby;
-  m[3] = ubx * ubx + T;
-  m[4] = ubx * uby;
-  m[5] = uby * uby + T;
-  m[6] = ubx * (u2 + 4.0 * T);
-  m[7] = uby * (u2 + 4.0 * T);
+  m[3] = fma(ubx, ubx, T);
+  m[4] = mul_rn(ubx, uby);
+  m[5] = fma(uby, uby, T);
+  m[6] = mul_rn(ubx, q);
+  m[7] = mul_rn(uby, q);
 }
 
 // p_i = exp(-(1 + lambda . P(xi_i))) for all 21 velocities (Eq. exponential / rho).
@@ -225,7 +234,7 @@ __device__ __forceinline__ void maxwellian_guess(double ubx, double uby, double 
 
 // exp(-(1 + lambda . P(xi_i))) for one velocity given at run time.
 __device__ __forceinline__ double exp_family_one(const double lam[NM], int cx, int cy) {
-  const double x = cx, y = cy, r2 = x * x + y * y;
+  const double x = cx, y = cy, r2 = cx * cx + cy * cy;
   double s = 1.0 + lam[0];
   s = fma(lam[1], x, s);
   s = fma(lam[2], y, s);
@@ -244,23 +253,28 @@ __device__ __forceinline__ double exp_family_one(const double lam[NM], int cx, i
 __device__ __forceinline__ void grad_phi(const Params& pr, double rho, double T, double cbx,
                                          double cby, const double du[2][2], const double dT[2],
                                          double* phi_f, double* phi_g, double* phi_q) {
-  const double mu = rho * pr.nu;
-  const double kappa = rho * pr.cp * pr.nu / pr.prandtl;
+  // two reciprocals serve all quotients (an FP64 division is some nine
+  // operations of the FP64 pipe)
+  const double iT = 1.0 / T, irho = 1.0 / rho;
+  const double mu = mul_rn(rho, pr.nu);
+  const double kappa = mul_rn(mul_rn(rho, pr.cp), pr.kappa_nu);
   const double div = du[0][0] + du[1][1];
-  const double sxx = -mu * (2.0 * du[0][0] - div);
-  const double syy = -mu * (2.0 * du[1][1] - div);
-  const double sxy = -mu * (du[0][1] + du[1][0]);
-  const double qx = -kappa * dT[0];
-  const double qy = -kappa * dT[1];
-  const double c2 = cbx * cbx + cby * cby;
-  const double qc = qx * cbx + qy * cby;
-  const double iT = 1.0 / T;
-  const double ps = (sxx * cbx * cbx + 2.0 * sxy * cbx * cby + syy * cby * cby) *
-                    (0.5 * iT * iT / rho);
-  const double pq = qc * (iT * iT / (rho * pr.cp)) * (0.5 * c2 * iT - pr.cp);
+  const double sxx = mul_rn(-mu, fma(2.0, du[0][0], -div));
+  const double syy = mul_rn(-mu, fma(2.0, du[1][1], -div));
+  const double sxy = mul_rn(-mu, du[0][1] + du[1][0]);
+  const double qx = mul_rn(-kappa, dT[0]);
+  const double qy = mul_rn(-kappa, dT[1]);
+  const double cxx = mul_rn(cbx, cbx), cyy = mul_rn(cby, cby);
+  const double c2 = cxx + cyy;
+  const double qc = fma(qx, cbx, mul_rn(qy, cby));
+  const double irc = mul_rn(irho, pr.icp);
+  const double iT2 = mul_rn(iT, iT);
+  const double ps = mul_rn(fma(sxx, cxx, fma(mul_rn(2.0, sxy), mul_rn(cbx, cby), mul_rn(syy, cyy))),
+                           mul_rn(mul_rn(0.5, iT2), irho));
+  const double pq = mul_rn(mul_rn(qc, mul_rn(iT2, irc)), fma(mul_rn(0.5, c2), iT, -pr.cp));
   *phi_f = ps + pq;
   *phi_q = pq;
-  *phi_g = 2.0 * qc / (rho * pr.cp);
+  *phi_g = mul_rn(mul_rn(2.0, qc), irc);
 }
 
 // Resolve a coordinate along one axis: periodic wrap or zero-gradient clamp.

@@ -11,45 +11,25 @@
 // Layout: structure of arrays. Plane p (f_0..f_20, g_0..g_20) of a buffer is
 // a contiguous nx*ny array, x fastest; lattice codes and moments likewise.
 // Each thread owns two columns of the block's dynamic shared memory: its 42
-// pulled populations (stride BLOCK) and the 21 FP64 equilibrium values per
-// unit density of its latest equilibrium solve (stride BLOCK).
+// pulled populations (stride BLOCK) and the 21 equilibrium values (64 bits
+// each) per unit density of its latest equilibrium solve (stride BLOCK).
 #include <type_traits>
 
 #include "alb_step.cuh"
 
 namespace alb {
 
-// Launch shape of the step kernel per precision: the FP32 form runs blocks of
-// 256 threads, two per SM (measured on the 4096^2 shear layer once developed,
-// through the batch kernel's compiled shapes: 620 MLUPS against 591 for
-// 128 x 4 and 555 for 128 x 3); FP64 plain runs 128 threads with up to 255
-// registers each.
-template <typename P>
-struct StepShape;
-template <>
-struct StepShape<float> {
-  static constexpr int B = 256, MINB = 2, LOG2B = 8;
-};
-template <>
-struct StepShape<double> {
-  static constexpr int B = 128, MINB = 1, LOG2B = 7;
-};
-
 // One time step of every node: block (bx, by) updates the tile of 2^lg nodes
 // along x by B >> lg rows at (bx << lg, by * (B >> lg)).
-template <typename P>
-__global__ void __launch_bounds__(StepShape<P>::B, StepShape<P>::MINB)
-    step_kernel(StepArgs<P> a, int lg) {
-  constexpr int B = StepShape<P>::B;
-  static_assert((1 << StepShape<P>::LOG2B) == B, "tiles of B nodes");
+template <typename P, int B, int MINB>
+__global__ void __launch_bounds__(B, MINB)
+    step_kernel(const __grid_constant__ StepArgs<P> a, int lg) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double s_tab[EXPT_N];
   __shared__ RebuildQueue<B> s_rq;
-  load_exptab(s_tab);  // includes a barrier
-  const Columns<P, B> cl(smem_raw);
+  const Columns<P, B> cl(smem_raw, s_tab);  // includes a barrier
   NodeCount nc;
-  tile_step<P, B>(a, blockIdx.x << lg, blockIdx.y << (StepShape<P>::LOG2B - lg), lg, cl, s_tab,
-                  s_rq, nc);
+  tile_step<P, B>(a, blockIdx.x << lg, blockIdx.y * (B >> lg), lg, cl, s_rq, nc);
   flush_counts(a.ctr, nc);
 }
 
@@ -80,11 +60,10 @@ __device__ __forceinline__ void init_prim(const double* rho, const double* rhoux
 // lattice chosen from the initial velocity, then the first collision.
 template <typename P>
 __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1))
-    init_kernel(InitArgs<P> a) {
+    init_kernel(const __grid_constant__ InitArgs<P> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double s_tab[EXPT_N];
-  load_exptab(s_tab);
-  const Columns<P, BLOCK> cl(smem_raw);
+  const Columns<P, BLOCK> cl(smem_raw, s_tab);
   const Params& pr = a.prm;
   const int x = blockIdx.x * BLOCK + threadIdx.x;
   const int y = blockIdx.y;
@@ -113,8 +92,9 @@ __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1)
     const int code = lat_code(U0x, U0y);
     P lam[NM];
     const bool realizable = (r > 0.0) && (T > 0.0) && isfinite(r) && isfinite(T);
-    const int ns = realizable ? node_equilibrium<P>(pr, ux - U0x, uy - U0y, T, s_tab, nullptr,
-                                                    cl.eq, lam, &cnt)
+    bool fixed = false;
+    const int ns = realizable ? node_equilibrium<P, BLOCK>(pr, cl, ux - U0x, uy - U0y, T, false,
+                                                           lam, &cnt, &fixed)
                               : NEWTON_UNREALIZABLE;
     if (!realizable) n_bad += 1;
     if (ns != NEWTON_OK && realizable) n_fail += 1;
@@ -127,7 +107,7 @@ __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1)
       double feq = 0.0;
       if (ns == NEWTON_OK) {
         grad_phi(pr, r, T, cbx, cby, du, dT, &phf, &phg, &phq);
-        feq = r * cl.eq[i * BLOCK];
+        feq = r * eq_f64<P>(cl.eq[i * BLOCK], fixed);
       }
       cl.pop[i * BLOCK] = (P)(feq * (1.0 + phf));
       cl.pop[(Q + i) * BLOCK] = (P)(gfac * feq * (1.0 + phg));
@@ -135,9 +115,6 @@ __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1)
     if (ns == NEWTON_OK) {
       // the first collision starts from the multipliers just found if the
       // flow starts its solves from previous multipliers
-      P wbuf[NM];
-#pragma unroll
-      for (int j = 0; j < NM; ++j) wbuf[j] = lam[j];
       // with the neighbourhood rule, the neighbours' initial lattices (Eq.
       // criterion on their initial velocities, boundary rule outside the grid)
       uint8_t nb[8];
@@ -154,8 +131,13 @@ __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1)
                                         select_shift(a.rhouy[kk] / rr, pr.n0, pr.umax));
           }
       }
-      collide_store<P, BLOCK>(pr, cl, code, k, a.ps, a.pop_out, a.mom_out, a.lat_out, a.nxt_out,
-                              s_tab, pr.warm ? wbuf : nullptr, a.lam_out, &cnt, &n_fail, nb);
+      const NodeState s = node_moments<P, BLOCK>(pr, cl, code, nb);
+      int n2 = NEWTON_UNREALIZABLE;
+      bool fixed2 = false;
+      if (s.rho > 0.0)
+        n2 = node_equilibrium<P, BLOCK>(pr, cl, s.ubx, s.uby, s.T, pr.warm, lam, &cnt, &fixed2);
+      node_store<P, BLOCK>(pr, cl, code, s, n2, fixed2, pr.warm, lam, k, a.ps, a.pop_out, a.mom_out,
+                           a.lat_out, a.nxt_out, a.lam_out, &n_fail);
     } else {
       for (int i = 0; i < NPLANES; ++i) a.pop_out[i * a.ps + k] = (P)0;
       a.mom_out[k] = (P)r;
@@ -221,14 +203,13 @@ __global__ void __launch_bounds__(BLOCK)
   double* eq = s_eq + threadIdx.x;
   double lam[NM];
   const double r = rho[k];
-  Params pr{};
-  pr.tol = tol;
-  pr.maxit = maxit;
   SolveCount cnt;
   int st = NEWTON_UNREALIZABLE;
   if (r > 0.0) {
     if (precision == 0) {
-      st = node_equilibrium<double>(pr, ubx[k], uby[k], T[k], s_tab, nullptr, eq, lam, &cnt);
+      int it = 0, ev = 0;
+      st = newton_fp64g(ubx[k], uby[k], T[k], tol, maxit, s_tab, eq, BLOCK, lam, &it, &ev, nullptr);
+      cnt.fp64_iters = it;
     } else {
       float l32[NM];  // the FP64 multipliers are asked for here
       st = equilibrium_mixed(ubx[k], uby[k], T[k], tol, maxit, s_tab, nullptr, eq, BLOCK, l32,
@@ -263,15 +244,20 @@ __global__ void select_kernel(const double* rho, const double* rhou, int n, doub
 
 static dim3 grid_of(const Params& p) { return dim3((p.nx + BLOCK - 1) / BLOCK, p.ny); }
 
-// Tiles of the step kernel: 2^lg nodes along x, the smallest power of two that
-// holds a row (at least 8, at most the block), and the block's other threads
-// on the following rows, so that narrow grids keep the threads busy.
-template <typename P>
-static dim3 step_grid(const Params& p, int* lg) {
+// Tiles of the step kernel: 2^lg nodes along x, the block's other threads on the
+// following rows. 32 nodes (one warp, one 128-byte line) along x rather than a
+// whole row: the pulls missing along an interface between two lattices then
+// share their senders within a tile, so each is solved fewer times and fewer
+// solves follow one another in one block (1021 x 733 shear layer: 0.089 against
+// 0.148 rebuild solves per node and 0.81 against 1.35 ms a step for rows of 256;
+// 64 wide 0.90 ms; 16 wide 0.80 ms there and 14.37 against 14.41 ms at 4096^2,
+// but half a line per row). Narrower or wider where the grid is.
+static dim3 step_grid(const Params& p, int block, int* lg) {
   int l = 3;
-  while (l < StepShape<P>::LOG2B && (1 << l) < p.nx) ++l;
+  while (l < 5 && (1 << l) < p.nx) ++l;
+  while ((1 << l) < block && (block >> l) >= 2 * p.ny) ++l;
   *lg = l;
-  const int rows = (1 << StepShape<P>::LOG2B) >> l;
+  const int rows = block >> l;
   return dim3((p.nx + (1 << l) - 1) >> l, (p.ny + rows - 1) / rows);
 }
 
@@ -301,26 +287,33 @@ cudaError_t launch_init(FlowDev& f, const double* rho, const double* rhoux, cons
   return cudaGetLastError();
 }
 
+template <typename P, int B, int MINB>
+static cudaError_t launch_step_shape(const FlowDev& f, cudaStream_t s) {
+  const cudaError_t e = allow_smem(step_kernel<P, B, MINB>, smem_bytes<P, B>());
+  if (e != cudaSuccess) return e;
+  int lg = 0;
+  const dim3 g = step_grid(f.prm, B, &lg);
+  step_kernel<P, B, MINB><<<g, B, smem_bytes<P, B>(), s>>>(step_args<P>(f, f.cur), lg);
+  return cudaGetLastError();
+}
+
+// Block size of the FP32 form: 256 threads, two blocks per SM. Smaller blocks
+// would fill more SMs on a small grid, but an interface tile has then fewer
+// threads for its rebuild solves, which are the longest chain of such a step
+// (64^2 vortex 0.146 ms against 0.153 with 128 and 0.180 with 64 threads,
+// 201^2 Riemann 0.151 / 0.161 / 0.207, 512^2 shear 0.31 / 0.42 / 0.58; blocks of
+// 512 measured 0.174, 0.166 and 0.345). Grids of fewer than 8 rows do not fill
+// the 32 x 8 tile: 128 threads (2048 x 4 tube 0.059 ms against 0.087).
 cudaError_t launch_step(FlowDev& f, cudaStream_t s) {
   if (f.q == 49) return launch_step_q49(f, s);
-  const int in = f.cur, out = f.cur ^ 1;
   cudaError_t e;
-  int lg = 0;
-  if (f.precision == 0) {
-    constexpr int B = StepShape<double>::B;
-    const StepArgs<double> a = step_args<double>(f, in);
-    const dim3 g = step_grid<double>(f.prm, &lg);
-    if ((e = allow_smem(step_kernel<double>, smem_bytes<double, B>())) != cudaSuccess) return e;
-    step_kernel<double><<<g, B, smem_bytes<double, B>(), s>>>(a, lg);
-  } else {
-    constexpr int B = StepShape<float>::B;
-    const StepArgs<float> a = step_args<float>(f, in);
-    const dim3 g = step_grid<float>(f.prm, &lg);
-    if ((e = allow_smem(step_kernel<float>, smem_bytes<float, B>())) != cudaSuccess) return e;
-    step_kernel<float><<<g, B, smem_bytes<float, B>(), s>>>(a, lg);
-  }
-  e = cudaGetLastError();
-  if (e == cudaSuccess) f.cur = out;
+  if (f.precision == 0)
+    e = launch_step_shape<double, 128, 1>(f, s);
+  else if (f.prm.ny >= 8)
+    e = launch_step_shape<float, 256, 2>(f, s);
+  else
+    e = launch_step_shape<float, 128, 4>(f, s);
+  if (e == cudaSuccess) f.cur ^= 1;
   return e;
 }
 

@@ -26,6 +26,7 @@
 #include <type_traits>
 
 #include "alb_device.cuh"
+#include "alb_fix.cuh"
 #include "exp_table.h"
 
 namespace alb {
@@ -75,6 +76,52 @@ __device__ __forceinline__ void visit_groups(const R l[NM], V& v, R base = (R)1)
   }
 }
 
+// The same groups as a loop over the speed a = 1, 2, 3 (pairs of the x and y
+// axis, and the diagonal quadruple for a < 3), for the passes of the FP32 form:
+// v.pair_x(g, k, s_+, s_-), v.pair_y(...) and v.quad(g, k, s_++, s_-+, s_--, s_+-)
+// with g = a - 1 and k the powers of a. The loop is kept rolled: the FP32 form's
+// node update is one long straight run of code per node, and instruction fetch
+// takes issue slots from it (23 % of the stalls at 2048^2 with the groups
+// unrolled).
+template <typename R>
+struct Pow {
+  R a, a2, a3;
+};
+template <typename R, typename V>
+__device__ __forceinline__ void visit_speeds(const R l[NM], V& v, R base) {
+  const R c = base + l[0];
+  v.rest(c);
+  const R l35 = l[3] + l[5];
+#pragma unroll 1
+  for (int g = 0; g < 3; ++g) {
+    Pow<R> k;
+    k.a = (R)(g + 1);
+    k.a2 = mul_rn(k.a, k.a);
+    k.a3 = mul_rn(k.a2, k.a);
+    {
+      const R ex = fma(k.a2, l[3], c), ox = fma(k.a3, l[6], mul_rn(k.a, l[1]));
+      v.pair_x(g, k, ex + ox, ex - ox);
+      const R ey = fma(k.a2, l[5], c), oy = fma(k.a3, l[7], mul_rn(k.a, l[2]));
+      v.pair_y(g, k, ey + oy, ey - oy);
+    }
+    if (g < 2) {
+      const R E = fma(k.a2, l35, c);
+      const R t3 = k.a3 + k.a3;
+      const R X = fma(t3, l[6], mul_rn(k.a, l[1])), Y = fma(t3, l[7], mul_rn(k.a, l[2]));
+      const R Z = mul_rn(k.a2, l[4]);
+      const R Ep = E + Z, Em = E - Z;
+      const R XpY = X + Y, XmY = X - Y;
+      v.quad(g, k, Ep + XpY, Em - XmY, Ep - XpY, Em + XmY);
+    }
+  }
+}
+// Index of a group's first point: pairs x: PX + 8 g (and + 2), pairs y: PY + 8 g
+// (and + 2), quadruples: PQ + 8 g .. + 3.
+constexpr int PX = 1, PY = 2, PQ = 5;
+static_assert(XI_X(PX + 16) == 3 && XI_X(PX + 18) == -3 && XI_Y(PY + 8) == 2 &&
+                  XI_Y(PY + 10) == -2 && XI_X(PQ + 9) == -2 && XI_Y(PQ + 11) == -2,
+              "index pattern of the velocity groups");
+
 // 2^(j/N), j = 0..N-1 (N = EXPT_N); kernels copy it to shared memory (lanes
 // index it freely).
 static __constant__ double c_exptab[EXPT_N] = {ALB_EXPT_TABLE_VALUES};
@@ -84,6 +131,15 @@ static __constant__ double c_exptab[EXPT_N] = {ALB_EXPT_TABLE_VALUES};
 __device__ __forceinline__ void load_exptab(double* s_tab) {
   for (int j = threadIdx.x; j < EXPT_N; j += blockDim.x) s_tab[j] = c_exptab[j];
   __syncthreads();
+}
+
+// 2^63 2^(-j/512): the fixed-point exponential's table (alb_fix.cuh), in global
+// memory (consecutive threads copy consecutive entries).
+static __device__ const uint64_t g_fixtab[FIXT_N] = {ALB_FIXT_TABLE_VALUES};
+
+// Copy it into a block's shared array of FIXT_N entries (all threads; no barrier).
+__device__ __forceinline__ void load_fixtab(uint64_t* s_fix) {
+  for (int j = threadIdx.x; j < FIXT_N; j += blockDim.x) s_fix[j] = g_fixtab[j];
 }
 
 // Exponent e = n >> 8 of the scale 2^(n/N) of the table exponentials below.
@@ -179,87 +235,124 @@ using dual::Exp2;
 // Packed lower triangle of the 8x8 Jacobian: entry (a, b), b <= a.
 __host__ __device__ constexpr int tri(int a, int b) { return a * (a + 1) / 2 + b; }
 
+// exp(v) for the FP32 Newton's passes: two instructions, relative error about
+// |v| 2^-24 + 2^-22, of the size that the FP32 rounding of the exponent itself
+// leaves; results below FP32's normal range are zero.
+__device__ __forceinline__ float exp_fast(float v) {
+  float r;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(mul_rn(v, 1.44269504f)));
+  return r;
+}
+
 // FP32 pass: F = sum p, G = sum p P and H = sum p P P^T at the visited
-// multipliers, accumulated group by group of the velocity set (compile-time
-// monomials).
+// multipliers. Every entry is a moment sum p x^m y^n with m + n <= 6. On this
+// velocity set it comes from 27 sums over the speeds a: of a symmetric pair's
+// sum (even powers of a) and difference (odd powers), and of a diagonal
+// quadruple's four parity combinations (even or odd in x and in y). They take
+// half the operations of accumulating G and H entry by entry, and half the
+// registers (36 + 9 accumulators spilled at 128 registers a thread).
 struct PassGH32 {
-  float Fs, Gs[NM], Hs[36];
+  float p0;
+  float X[7], Y[7];      // pairs: sum a^n (p+ + p-) for even n, (p+ - p-) for odd n
+  float E[7], O[7];      // quadruples: even/even (n even); x odd (n odd), x and y odd (n even)
+  float Py[7];           // quadruples: y odd (n odd)
   __device__ __forceinline__ PassGH32() {
-    Fs = 0.0f;
+    p0 = 0.0f;
 #pragma unroll
-    for (int k = 0; k < NM; ++k) Gs[k] = 0.0f;
-#pragma unroll
-    for (int k = 0; k < 36; ++k) Hs[k] = 0.0f;
+    for (int n = 0; n < 7; ++n) X[n] = Y[n] = E[n] = O[n] = Py[n] = 0.0f;
   }
-  template <int I>
-  __device__ __forceinline__ void point(float p) {
-    Fs += p;
-#pragma unroll
-    for (int a = 0; a < NM; ++a) {
-      Gs[a] = madd(Gs[a], p, PM(a, I));
-#pragma unroll
-      for (int b = 0; b <= a; ++b) Hs[tri(a, b)] = madd(Hs[tri(a, b)], p, PM(a, I) * PM(b, I));
-    }
+  __device__ __forceinline__ void rest(float s) { p0 = exp_fast(-s); }
+  static __device__ __forceinline__ void add_pair(float M[7], const Pow<float>& k, float pp,
+                                                  float pm) {
+    const float S = pp + pm, D = mul_rn(k.a, pp - pm);
+    const float S2 = mul_rn(k.a2, S), D3 = mul_rn(k.a2, D);
+    M[0] += S;
+    M[1] += D;
+    M[2] += S2;
+    M[3] += D3;
+    M[4] = fmaf(k.a2, S2, M[4]);
+    M[5] = fmaf(k.a2, D3, M[5]);
+    M[6] = fmaf(mul_rn(k.a2, k.a2), S2, M[6]);
   }
-  __device__ __forceinline__ void rest(float s) { point<0>(expf(-s)); }
-  // A symmetric pair enters through the sum S and difference D of its two
-  // points: every sum takes c S or c D, with c the compile-time value of the
-  // monomial (product) at the first point and D where the second point flips
-  // its sign (the grouping of the FP64 Jacobian, jac_pair).
-  template <int A, int AX, int IP, int IM>
-  __device__ __forceinline__ void pair(float sp, float sm) {
-    const float pp = expf(-sp), pm = expf(-sm);
-    const float S = pp + pm, D = pp - pm;
-    Fs += S;
-#pragma unroll
-    for (int a = 0; a < NM; ++a) {
-      const int ca = PM(a, IP);
-      if (ca != 0) Gs[a] = madd(Gs[a], PM(a, IM) == ca ? S : D, ca);
-#pragma unroll
-      for (int b = 0; b <= a; ++b) {
-        const int c = PM(a, IP) * PM(b, IP);
-        if (c != 0) Hs[tri(a, b)] = madd(Hs[tri(a, b)], PM(a, IM) * PM(b, IM) == c ? S : D, c);
-      }
-    }
+  __device__ __forceinline__ void pair_x(int, const Pow<float>& k, float sp, float sm) {
+    add_pair(X, k, exp_fast(-sp), exp_fast(-sm));
   }
-  // A diagonal quadruple enters through its four parity combinations (even
-  // or odd in x, even or odd in y), as in jac_quad.
-  template <int A, int IPP, int IMP, int IMM, int IPM>
-  __device__ __forceinline__ void quad(float spp, float smp, float smm, float spm) {
-    const float ppp = expf(-spp), pmp = expf(-smp), pmm = expf(-smm), ppm = expf(-spm);
+  __device__ __forceinline__ void pair_y(int, const Pow<float>& k, float sp, float sm) {
+    add_pair(Y, k, exp_fast(-sp), exp_fast(-sm));
+  }
+  __device__ __forceinline__ void quad(int, const Pow<float>& k, float spp, float smp, float smm,
+                                       float spm) {
+    const float ppp = exp_fast(-spp), pmp = exp_fast(-smp), pmm = exp_fast(-smm), ppm = exp_fast(-spm);
     const float Ap = ppp + ppm, Bm = pmp + pmm, Cp = ppp - ppm, Dm = pmp - pmm;
-    const float ee = Ap + Bm, oe = Ap - Bm, eo = Cp + Dm, oo = Cp - Dm;
-    Fs += ee;
-#pragma unroll
-    for (int a = 0; a < NM; ++a) {
-      const int ca = PM(a, IPP);
-      if (ca != 0) {
-        const bool xo = PM(a, IMP) == -ca, yo = PM(a, IPM) == -ca;
-        Gs[a] = madd(Gs[a], xo ? (yo ? oo : oe) : (yo ? eo : ee), ca);
-      }
-#pragma unroll
-      for (int b = 0; b <= a; ++b) {
-        const int c = PM(a, IPP) * PM(b, IPP);
-        if (c == 0) continue;
-        const bool xo = PM(a, IMP) * PM(b, IMP) == -c;  // x -> -x flips the sign
-        const bool yo = PM(a, IPM) * PM(b, IPM) == -c;  // y -> -y flips the sign
-        Hs[tri(a, b)] = madd(Hs[tri(a, b)], xo ? (yo ? oo : oe) : (yo ? eo : ee), c);
-      }
-    }
+    const float a4 = mul_rn(k.a2, k.a2);
+    const float ee = Ap + Bm, oe = mul_rn(k.a, Ap - Bm), eo = mul_rn(k.a, Cp + Dm);
+    const float oo = mul_rn(k.a2, Cp - Dm), e2 = mul_rn(k.a2, ee);
+    E[0] += ee;
+    E[2] += e2;
+    E[4] = fmaf(k.a2, e2, E[4]);
+    E[6] = fmaf(a4, e2, E[6]);
+    O[1] += oe;
+    O[3] = fmaf(k.a2, oe, O[3]);
+    O[5] = fmaf(a4, oe, O[5]);
+    Py[1] += eo;
+    Py[3] = fmaf(k.a2, eo, Py[3]);
+    Py[5] = fmaf(a4, eo, Py[5]);
+    O[2] += oo;
+    O[4] = fmaf(k.a2, oo, O[4]);
+    O[6] = fmaf(a4, oo, O[6]);
   }
-  __device__ __forceinline__ float F() const { return Fs; }
+  __device__ __forceinline__ float F() const { return p0 + X[0] + Y[0] + E[0]; }
   __device__ __forceinline__ void scale(float z) {
-    Fs *= z;
+    p0 = mul_rn(p0, z);
 #pragma unroll
-    for (int k = 0; k < NM; ++k) Gs[k] *= z;
-#pragma unroll
-    for (int k = 0; k < 36; ++k) Hs[k] *= z;
+    for (int n = 0; n < 7; ++n) {
+      X[n] = mul_rn(X[n], z);
+      Y[n] = mul_rn(Y[n], z);
+      E[n] = mul_rn(E[n], z);
+      O[n] = mul_rn(O[n], z);
+      Py[n] = mul_rn(Py[n], z);
+    }
   }
   __device__ __forceinline__ void assemble(float G[NM], float H[36]) const {
+    const float x3 = X[3] + O[3], y3 = Y[3] + Py[3];    // x^3, y^3
+    G[0] = F();
+    G[1] = X[1] + O[1];
+    G[2] = Y[1] + Py[1];
+    G[3] = X[2] + E[2];
+    G[4] = O[2];
+    G[5] = Y[2] + E[2];
+    G[6] = x3 + O[3];                                   // x^3 + x y^2
+    G[7] = y3 + Py[3];
 #pragma unroll
-    for (int k = 0; k < NM; ++k) G[k] = Gs[k];
-#pragma unroll
-    for (int k = 0; k < 36; ++k) H[k] = Hs[k];
+    for (int k = 0; k < NM; ++k) H[tri(k, 0)] = G[k];
+    H[tri(1, 1)] = G[3];
+    H[tri(2, 1)] = G[4];
+    H[tri(2, 2)] = G[5];
+    H[tri(3, 1)] = x3;
+    H[tri(3, 2)] = Py[3];
+    H[tri(3, 3)] = X[4] + E[4];
+    H[tri(4, 1)] = Py[3];
+    H[tri(4, 2)] = O[3];
+    H[tri(4, 3)] = O[4];
+    H[tri(4, 4)] = E[4];
+    H[tri(5, 1)] = O[3];
+    H[tri(5, 2)] = y3;
+    H[tri(5, 3)] = E[4];
+    H[tri(5, 4)] = O[4];
+    H[tri(5, 5)] = Y[4] + E[4];
+    H[tri(6, 1)] = fmaf(2.0f, E[4], X[4]);
+    H[tri(6, 2)] = 2.0f * O[4];
+    H[tri(6, 3)] = fmaf(2.0f, O[5], X[5]);
+    H[tri(6, 4)] = 2.0f * Py[5];
+    H[tri(6, 5)] = 2.0f * O[5];
+    H[tri(6, 6)] = fmaf(4.0f, E[6], X[6]);
+    H[tri(7, 1)] = 2.0f * O[4];
+    H[tri(7, 2)] = fmaf(2.0f, E[4], Y[4]);
+    H[tri(7, 3)] = 2.0f * Py[5];
+    H[tri(7, 4)] = 2.0f * O[5];
+    H[tri(7, 5)] = fmaf(2.0f, Py[5], Y[5]);
+    H[tri(7, 6)] = 4.0f * O[6];
+    H[tri(7, 7)] = fmaf(4.0f, E[6], Y[6]);
   }
 };
 
@@ -406,6 +499,120 @@ struct PassMul64 : SumsG64 {
   }
 };
 
+// Exponents in Q25 octaves (alb_fix.cuh); visit_speeds runs on them unchanged.
+// Arithmetic modulo 2^32; the operators live in a namespace of their own, found
+// by argument-dependent lookup.
+namespace fixe {
+struct Oct {
+  uint32_t v;
+  Oct() = default;
+  __device__ __forceinline__ explicit Oct(int c) : v((uint32_t)c) {}
+};
+__device__ __forceinline__ Oct oct(uint32_t v) {
+  Oct o;
+  o.v = v;
+  return o;
+}
+__device__ __forceinline__ Oct operator+(Oct a, Oct b) { return oct(a.v + b.v); }
+__device__ __forceinline__ Oct operator-(Oct a, Oct b) { return oct(a.v - b.v); }
+__device__ __forceinline__ Oct mul_rn(Oct a, Oct b) { return oct(a.v * b.v); }
+__device__ __forceinline__ Oct fma(Oct a, Oct b, Oct c) { return oct(a.v * b.v + c.v); }
+}  // namespace fixe
+using fixe::Oct;
+
+// Q63 constraint sums over the groups of the velocity set, started at -m
+// (modulo 2^64), so that they end as the residual G = sum p P - m: the grouping
+// of SumsG64. A weighted term is one 32 x 32 + 64 multiply-add and one 32-bit one.
+struct SumsFix {
+  uint64_t M[NM];
+  __device__ __forceinline__ explicit SumsFix(const uint64_t mneg[NM]) {
+#pragma unroll
+    for (int k = 0; k < NM; ++k) M[k] = mneg[k];
+  }
+  __device__ __forceinline__ void add_rest(uint64_t p) { M[0] += p; }
+  template <int AX>
+  __device__ __forceinline__ void add_pair(int g, uint64_t pp, uint64_t pm) {
+    const uint32_t a = g + 1;
+    const uint64_t S = pp + pm, D = pp - pm;
+    M[0] += S;
+    M[AX == 0 ? 1 : 2] += a * D;
+    M[AX == 0 ? 3 : 5] += (a * a) * S;
+    M[AX == 0 ? 6 : 7] += (a * a * a) * D;
+  }
+  __device__ __forceinline__ void add_quad(int g, uint64_t ppp, uint64_t pmp, uint64_t pmm,
+                                           uint64_t ppm) {
+    const uint32_t a = g + 1;
+    const uint64_t Ap = ppp + ppm, Bm = pmp + pmm;  // sx = +1, sx = -1
+    const uint64_t Cp = ppp - ppm, Dm = pmp - pmm;
+    const uint64_t sum = Ap + Bm, xs = Ap - Bm, ys = Cp + Dm, xys = Cp - Dm;
+    M[0] += sum;
+    M[1] += a * xs;
+    M[2] += a * ys;
+    M[3] += (a * a) * sum;
+    M[4] += (a * a) * xys;
+    M[5] += (a * a) * sum;
+    M[6] += (2 * a * a * a) * xs;
+    M[7] += (2 * a * a * a) * ys;
+  }
+};
+
+// Evaluation: Q63 populations of the exponents into the column, their sums, and
+// the largest exponent (as an unsigned number, so that one below zero shows
+// too).
+struct PassFix : SumsFix {
+  const uint64_t* tab;
+  uint64_t* col;
+  int stride;
+  uint32_t ymax;
+  __device__ __forceinline__ PassFix(const uint64_t* t, uint64_t* c, int s, const uint64_t mneg[NM])
+      : SumsFix(mneg), tab(t), col(c), stride(s), ymax(0) {}
+  __device__ __forceinline__ uint64_t ex(int i, Oct y) {
+    ymax = ymax > y.v ? ymax : y.v;
+    const uint64_t p = fix_exp(y.v, tab);
+    col[(size_t)i * stride] = p;
+    return p;
+  }
+  __device__ __forceinline__ void rest(Oct y) { add_rest(ex(0, y)); }
+  __device__ __forceinline__ void pair_x(int g, const Pow<Oct>&, Oct p, Oct m) {
+    add_pair<0>(g, ex(PX + 8 * g, p), ex(PX + 2 + 8 * g, m));
+  }
+  __device__ __forceinline__ void pair_y(int g, const Pow<Oct>&, Oct p, Oct m) {
+    add_pair<1>(g, ex(PY + 8 * g, p), ex(PY + 2 + 8 * g, m));
+  }
+  __device__ __forceinline__ void quad(int g, const Pow<Oct>&, Oct pp, Oct mp, Oct mm, Oct pm) {
+    add_quad(g, ex(PQ + 8 * g, pp), ex(PQ + 1 + 8 * g, mp), ex(PQ + 2 + 8 * g, mm),
+             ex(PQ + 3 + 8 * g, pm));
+  }
+};
+
+// Multiplicative pass after a small step dl of the multipliers, in place in the
+// column: p_i <- p_i exp(-d_i), d_i = dl . P(xi_i) in FP32, and the sums again
+// (the fixed-point form of PassMul64).
+struct PassMulFix : SumsFix {
+  uint64_t* col;
+  int stride;
+  FixStep fs;
+  __device__ __forceinline__ PassMulFix(uint64_t* c, int s, const uint64_t mneg[NM], float bound)
+      : SumsFix(mneg), col(c), stride(s), fs(fix_step(bound)) {}
+  __device__ __forceinline__ uint64_t upd(int i, float d) const {
+    uint64_t* q = col + (size_t)i * stride;
+    const uint64_t p = fix_scale(*q, d, fs);
+    *q = p;
+    return p;
+  }
+  __device__ __forceinline__ void rest(float d) { add_rest(upd(0, d)); }
+  __device__ __forceinline__ void pair_x(int g, const Pow<float>&, float p, float m) {
+    add_pair<0>(g, upd(PX + 8 * g, p), upd(PX + 2 + 8 * g, m));
+  }
+  __device__ __forceinline__ void pair_y(int g, const Pow<float>&, float p, float m) {
+    add_pair<1>(g, upd(PY + 8 * g, p), upd(PY + 2 + 8 * g, m));
+  }
+  __device__ __forceinline__ void quad(int g, const Pow<float>&, float pp, float mp, float mm, float pm) {
+    add_quad(g, upd(PQ + 8 * g, pp), upd(PQ + 1 + 8 * g, mp), upd(PQ + 2 + 8 * g, mm),
+             upd(PQ + 3 + 8 * g, pm));
+  }
+};
+
 // Cholesky factor of the Jacobian, FP32: the packed lower triangle L with the
 // reciprocals of its diagonal entries in the diagonal slots, so that the
 // solves multiply. No diagonal (Jacobi) scaling: the backward error of the
@@ -415,6 +622,13 @@ struct Fact32 {
   float L[36];
 };
 
+// Approximate reciprocal square root without the handling of subnormal inputs.
+__device__ __forceinline__ float rsqrt_fast(float v) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(v));
+  return r;
+}
+
 __device__ __forceinline__ bool factor32(const float H[36], Fact32& fc) {
   bool ok = true;
 #pragma unroll
@@ -423,14 +637,14 @@ __device__ __forceinline__ bool factor32(const float H[36], Fact32& fc) {
 #pragma unroll
     for (int k = 0; k < j; ++k) dj = fmaf(-fc.L[tri(j, k)], fc.L[tri(j, k)], dj);
     ok = ok && (dj > 0.0f);
-    const float il = rsqrtf(fmaxf(dj, 1e-30f));
+    const float il = rsqrt_fast(fmaxf(dj, 1e-30f));
     fc.L[tri(j, j)] = il;
 #pragma unroll
     for (int i = j + 1; i < NM; ++i) {
       float s = H[tri(i, j)];
 #pragma unroll
       for (int k = 0; k < j; ++k) s = fmaf(-fc.L[tri(i, k)], fc.L[tri(j, k)], s);
-      fc.L[tri(i, j)] = s * il;
+      fc.L[tri(i, j)] = mul_rn(s, il);
     }
   }
   return ok;
@@ -444,14 +658,14 @@ __device__ __forceinline__ void solve32(const Fact32& fc, const float g[NM], flo
     float s = g[i];
 #pragma unroll
     for (int k = 0; k < i; ++k) s = fmaf(-fc.L[tri(i, k)], y[k], s);
-    y[i] = s * fc.L[tri(i, i)];
+    y[i] = mul_rn(s, fc.L[tri(i, i)]);
   }
 #pragma unroll
   for (int i = NM - 1; i >= 0; --i) {
     float s = y[i];
 #pragma unroll
     for (int k = i + 1; k < NM; ++k) s = fmaf(-fc.L[tri(k, i)], y[k], s);
-    y[i] = s * fc.L[tri(i, i)];
+    y[i] = mul_rn(s, fc.L[tri(i, i)]);
   }
 #pragma unroll
   for (int i = 0; i < NM; ++i) dl[i] = y[i];
@@ -463,103 +677,116 @@ __device__ __forceinline__ void solve32(const Fact32& fc, const float g[NM], flo
 // point of the Newton iteration after a change of lattice.
 template <typename R>
 __device__ __forceinline__ void shift_multipliers(const R l[NM], R dx, R dy, R o[NM]) {
-  const R d2 = dx * dx + dy * dy;
-  o[0] = l[0] - l[1] * dx - l[2] * dy + l[3] * dx * dx + l[4] * dx * dy + l[5] * dy * dy -
-         l[6] * dx * d2 - l[7] * dy * d2;
-  o[1] = l[1] - (R)2 * l[3] * dx - l[4] * dy + l[6] * ((R)3 * dx * dx + dy * dy) +
-         (R)2 * l[7] * dx * dy;
-  o[2] = l[2] - l[4] * dx - (R)2 * l[5] * dy + (R)2 * l[6] * dx * dy +
-         l[7] * (dx * dx + (R)3 * dy * dy);
-  o[3] = l[3] - (R)3 * l[6] * dx - l[7] * dy;
-  o[4] = l[4] - (R)2 * l[6] * dy - (R)2 * l[7] * dx;
-  o[5] = l[5] - l[6] * dx - (R)3 * l[7] * dy;
+  // (dx, dy and their products are small integers, exact)
+  const R xx = mul_rn(dx, dx), xy = mul_rn(dx, dy), yy = mul_rn(dy, dy), d2 = xx + yy;
+  const R x3 = fma((R)2, xx, d2), y3 = fma((R)2, yy, d2);
+  R t = fma(-l[1], dx, l[0]);
+  t = fma(-l[2], dy, t);
+  t = fma(l[3], xx, t);
+  t = fma(l[4], xy, t);
+  t = fma(l[5], yy, t);
+  t = fma(-l[6], mul_rn(dx, d2), t);
+  o[0] = fma(-l[7], mul_rn(dy, d2), t);
+  t = fma(mul_rn((R)-2, l[3]), dx, l[1]);
+  t = fma(-l[4], dy, t);
+  t = fma(l[6], x3, t);
+  o[1] = fma(mul_rn((R)2, l[7]), xy, t);
+  t = fma(-l[4], dx, l[2]);
+  t = fma(mul_rn((R)-2, l[5]), dy, t);
+  t = fma(mul_rn((R)2, l[6]), xy, t);
+  o[2] = fma(l[7], y3, t);
+  o[3] = fma(-l[7], dy, fma(mul_rn((R)-3, l[6]), dx, l[3]));
+  o[4] = fma(mul_rn((R)-2, l[7]), dx, fma(mul_rn((R)-2, l[6]), dy, l[4]));
+  o[5] = fma(mul_rn((R)-3, l[7]), dy, fma(-l[6], dx, l[5]));
   o[6] = l[6];
   o[7] = l[7];
 }
 
 // FP32 phase: damped Newton from lam (warm start) or, if warm is false, from
 // the Maxwellian; on success fc holds the factor of the Jacobian at the
-// returned multipliers. Returns NEWTON_OK or NEWTON_SINGULAR (non-finite
-// values or a non-positive pivot).
+// returned multipliers or one near step before them. Returns NEWTON_OK or
+// NEWTON_SINGULAR (non-finite values or a non-positive pivot).
 //
 // Written as one loop with a single evaluation pass and a single
-// factorisation, so that the unrolled pass (21 exponentials and the 44 sums)
-// exists once in the code: each turn evaluates the point `lc` and then acts
-// on it according to why it was evaluated (a start, a line-search trial, the
-// full step taken near the root). The points evaluated and the steps
-// accepted are those of the plain formulation: start, then per Newton step
-// the factor and direction at the accepted point and an Armijo line search.
-static __device__ __noinline__ int newton_fp32(float ubx, float uby, float T, int maxit, bool warm,
-                                               float lam[NM], Fact32& fc, int* iters) {
-  enum { START_WARM, START_MAXWELL, TRIAL, FULL_STEP };
+// factorisation, so that the pass exists once in the code: each turn evaluates
+// the point lam and then acts on it according to why it was evaluated (a
+// start, a line-search trial, the point a failed line search returns to).
+//
+// Inlined into each solver (once), so that the factor stays in registers
+// between this phase and the refinement. What is live across a pass is kept
+// small for the same reason: the last step's direction and length but not its
+// start, and the three inputs instead of the eight targets. *gres is the
+// residual maximum (FP32) at the last evaluated point.
+__device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int maxit, bool warm,
+                                           float lam[NM], Fact32& fc, int* iters, float* gres) {
+  enum { START_WARM, START_MAXWELL, TRIAL, RETURNED };
   *iters = 0;
-  float m[NM];
-  {
-    const float u2 = ubx * ubx + uby * uby;
-    m[0] = 1.0f; m[1] = ubx; m[2] = uby;
-    m[3] = fmaf(ubx, ubx, T); m[4] = ubx * uby; m[5] = fmaf(uby, uby, T);
-    m[6] = ubx * fmaf(4.0f, T, u2); m[7] = uby * fmaf(4.0f, T, u2);
-  }
-  auto dual = [&](const float* l, float F) {
-#pragma unroll
-    for (int k = 0; k < NM; ++k) F = fmaf(l[k], m[k], F);
-    return F;
-  };
   // Maxwellian multipliers with lambda_0 = 0 (fixed from the normalisation
   // once evaluated)
-  auto maxwell = [&](float* l) {
+  auto maxwell = [&]() {
     const float iT = 1.0f / T;
 #pragma unroll
-    for (int k = 0; k < NM; ++k) l[k] = 0.0f;
-    l[1] = -ubx * iT;
-    l[2] = -uby * iT;
-    l[3] = 0.5f * iT;
-    l[5] = 0.5f * iT;
+    for (int k = 0; k < NM; ++k) lam[k] = 0.0f;
+    lam[1] = mul_rn(-ubx, iT);
+    lam[2] = mul_rn(-uby, iT);
+    lam[3] = mul_rn(0.5f, iT);
+    lam[5] = lam[3];
   };
-  float lc[NM], dl[NM];
   int mode = START_WARM;
-  if (warm) {
-#pragma unroll
-    for (int k = 0; k < NM; ++k) lc[k] = lam[k];
-  } else {
-    maxwell(lc);
+  if (!warm) {
+    maxwell();
     mode = START_MAXWELL;
   }
+  float dl[NM];
   float Fd = 0.0f, gd = 0.0f, t = 1.0f;
   int it = 0, ls = 0;
+#pragma unroll 1
   for (;;) {
     PassGH32 pc;
-    visit_groups<float>(lc, pc);
+    visit_speeds<float>(lam, pc, 1.0f);
     float F = pc.F();
     if (mode == START_WARM) {
       if (!(isfinite(F) && F > 0.0f)) {
-        maxwell(lc);
+        maxwell();
         mode = START_MAXWELL;
         continue;
       }
     } else if (mode == START_MAXWELL) {
       // the pass at lambda_0 = 0 gives Z = F; all its sums scale by 1/Z
       const float iz = 1.0f / F;
-      lc[0] = logf(F);
+      lam[0] = logf(F);
       pc.scale(iz);
       F = pc.F();
-    } else if (mode == TRIAL) {
-      const float Fc = dual(lc, F);
-      if (!(isfinite(Fc) && Fc <= Fd - 1e-4f * t * gd + 4e-7f * fabsf(Fd))) {
-        t *= 0.5f;
-        if (++ls >= 12) break;  // no acceptable step: fc is the factor at lam
+    }
+    // targets, formed again in every turn (the empty statement keeps the
+    // compiler from carrying them across the pass)
+    float ux = ubx, uy = uby, Tt = T;
+    asm volatile("" : "+f"(ux), "+f"(uy), "+f"(Tt));
+    float m[NM];
+    {
+      const float u2 = fmaf(ux, ux, mul_rn(uy, uy)), q = fmaf(4.0f, Tt, u2);
+      m[0] = 1.0f; m[1] = ux; m[2] = uy;
+      m[3] = fmaf(ux, ux, Tt); m[4] = mul_rn(ux, uy); m[5] = fmaf(uy, uy, Tt);
+      m[6] = mul_rn(ux, q); m[7] = mul_rn(uy, q);
+    }
 #pragma unroll
-        for (int k = 0; k < NM; ++k) lc[k] = fmaf(t, dl[k], lam[k]);
+    for (int k = 0; k < NM; ++k) F = fmaf(lam[k], m[k], F);  // the dual
+    if (mode == TRIAL) {
+      if (!(isfinite(F) && F <= fmaf(4e-7f, fabsf(Fd), fmaf(mul_rn(-1e-4f, t), gd, Fd)))) {
+        // halve the step; with no acceptable one, back to its start for the
+        // factor there
+        const bool back = ++ls >= 12;
+        const float dt = back ? t : mul_rn(0.5f, t);
+#pragma unroll
+        for (int k = 0; k < NM; ++k) lam[k] = fmaf(-dt, dl[k], lam[k]);
+        t -= dt;
+        if (back) mode = RETURNED;
         continue;
       }
       ++it;
-    } else if (!isfinite(F)) {  // FULL_STEP
-      return NEWTON_SINGULAR;
     }
     // accepted point: the Newton step there
-#pragma unroll
-    for (int k = 0; k < NM; ++k) lam[k] = lc[k];
-    Fd = dual(lam, F);
+    Fd = F;
     float G[NM], H[36];
     pc.assemble(G, H);
     float gmax = 0.0f;
@@ -568,33 +795,33 @@ static __device__ __noinline__ int newton_fp32(float ubx, float uby, float T, in
       G[k] -= m[k];
       gmax = fmaxf(gmax, fabsf(G[k]));
     }
+    *gres = gmax;
     if (!isfinite(gmax) || !factor32(H, fc)) return NEWTON_SINGULAR;
     // FP32 exit at 1e-6, five times the FP32 residual's own noise (about
-    // 2e-7): below that the FP32 steps only chase rounding, and the FP64
+    // 2e-7): below that the FP32 steps only chase rounding, and the
     // refinement contracts by about 1e-4 per residual from either level
-    if (mode == FULL_STEP || gmax <= 1e-6f || it >= maxit) break;
+    if (mode == RETURNED || gmax <= 1e-6f || it >= maxit) break;
     solve32(fc, G, dl);
     gd = 0.0f;
 #pragma unroll
     for (int k = 0; k < NM; ++k) gd = fmaf(G[k], dl[k], gd);
     if (!(gd > 0.0f)) break;
 #pragma unroll
-    for (int k = 0; k < NM; ++k) lc[k] = lam[k] + dl[k];
-    if (gd <= 2e-6f * fmaxf(1.0f, fabsf(Fd))) {
+    for (int k = 0; k < NM; ++k) lam[k] += dl[k];
+    if (gd <= mul_rn(2e-6f, fmaxf(1.0f, fabsf(Fd)))) {
       // The predicted decrease gd/2 of the dual lies below its FP32 resolution:
       // a line search would only compare rounding noise. This close to the root
-      // the full Newton step is safe; take it and leave the rest to the FP64
-      // refinement. The refinement contracts by about |I - H32^-1 H| per
-      // residual, so it gets the factor of the Jacobian at the new multipliers
-      // (one more FP32 pass): a factor one step old costs about one more FP64
-      // residual per solve.
-      mode = FULL_STEP;
+      // the full Newton step is safe; take it and leave the rest to the
+      // refinement, with the factor of the point before it: the exponents moved
+      // by some 1e-3, so it still contracts by about that per residual, at
+      // 0.6 more residuals a solve than with a fresh factor but without the
+      // pass and the factorisation that one takes.
       ++it;
-    } else {
-      mode = TRIAL;
-      t = 1.0f;
-      ls = 0;
+      break;
     }
+    mode = TRIAL;
+    t = 1.0f;
+    ls = 0;
   }
   *iters = it;
   return NEWTON_OK;
@@ -613,8 +840,10 @@ static_assert(pm_max(0) == 1 && pm_max(1) == 3 && pm_max(2) == 3 && pm_max(3) ==
                   pm_max(4) == 4 && pm_max(5) == 9 && pm_max(6) == 27 && pm_max(7) == 27,
               "monomial bounds of the D2Q21 set");
 __device__ __forceinline__ float step_exponent_bound(const float dl[NM]) {
-  return fabsf(dl[0]) + 3.0f * (fabsf(dl[1]) + fabsf(dl[2])) + 4.0f * fabsf(dl[4]) +
-         9.0f * (fabsf(dl[3]) + fabsf(dl[5])) + 27.0f * (fabsf(dl[6]) + fabsf(dl[7]));
+  float b = fmaf(3.0f, fabsf(dl[1]) + fabsf(dl[2]), fabsf(dl[0]));
+  b = fmaf(4.0f, fabsf(dl[4]), b);
+  b = fmaf(9.0f, fabsf(dl[3]) + fabsf(dl[5]), b);
+  return fmaf(27.0f, fabsf(dl[6]) + fabsf(dl[7]), b);
 }
 
 // FP64 refinement: lambda <- lambda + H32^-1 G64(lambda) until max|G|/rho <= tol.
@@ -705,6 +934,12 @@ static __device__ __noinline__ int refine_fp64(double ubx, double uby, double T,
 // Work counts of one equilibrium solve.
 struct SolveCount {
   unsigned fp32_iters = 0, fp64_evals = 0, fp64_iters = 0, fp64_updates = 0;
+  __device__ __forceinline__ void add(const SolveCount& o) {
+    fp32_iters += o.fp32_iters;
+    fp64_evals += o.fp64_evals;
+    fp64_iters += o.fp64_iters;
+    fp64_updates += o.fp64_updates;
+  }
 };
 
 // Jacobian H = sum_i p_i P(xi_i) P(xi_i)^T (packed lower triangle) from the
@@ -1049,30 +1284,131 @@ static __device__ __noinline__ int newton4_fp64g(double ubx, double uby, double 
   }
 }
 
-// Equilibrium of the FP32 form: FP32 Newton (from the warm start if given,
-// else from the Maxwellian; again from the Maxwellian if the warm start
-// fails), FP64 refinement, full FP64 Newton as the last fallback. The FP64
-// equilibrium per unit density lands in col[i * stride]; the multipliers in
-// lam32 (FP32, as the warm start keeps them) and, if lam64 is given, in FP64.
-__device__ __forceinline__ int equilibrium_mixed(double ubx, double uby, double T, double tol,
-                                                 int maxit, const double* tab, const float* warm,
-                                                 double* col, int stride, float lam32[NM],
-                                                 double* lam64, SolveCount* cnt) {
+// Largest exponent |1 + lambda . P(xi_i)| over the velocities is at most this:
+// the larger of the axis and the diagonal velocities' bounds.
+__device__ __forceinline__ float exponent_bound(const float l[NM]) {
+  const float ax = fmaf(9.0f, fabsf(l[3]), fmaf(3.0f, fabsf(l[1]), mul_rn(27.0f, fabsf(l[6]))));
+  const float ay = fmaf(9.0f, fabsf(l[5]), fmaf(3.0f, fabsf(l[2]), mul_rn(27.0f, fabsf(l[7]))));
+  const float dg = fmaf(4.0f, fabsf(l[3]) + fabsf(l[4]) + fabsf(l[5]),
+                        fmaf(2.0f, fabsf(l[1]) + fabsf(l[2]),
+                             mul_rn(16.0f, fabsf(l[6]) + fabsf(l[7]))));
+  return fabsf(1.0f + l[0]) + fmaxf(fmaxf(ax, ay), dg);
+}
+
+// Refinement of the FP32 form in fixed point: as refine_fp64, lambda <- lambda +
+// H32^-1 G(lambda) until max|G|/rho <= tol with G the exact sum of the
+// populations in the column, here in Q63 (alb_fix.cuh). Returns NEWTON_OK with
+// the Q63 populations in col[i * stride], or another status for the states it
+// does not take (an exponent outside the fixed-point range, FP32 residual above
+// 1/64: the Q63 residual has to stay below one) and for failures; the caller
+// then refines in FP64.
+__device__ __forceinline__ int refine_fix(double ubx, double uby, double T, float tolf, int maxr,
+                                          float lam[NM], const Fact32& fc, float gres,
+                                          const uint64_t* tab, uint64_t* col, int stride,
+                                          int* evals, int* updates) {
+  *evals = 0;
+  *updates = 0;
+  if (!(gres < 0.015625f)) return NEWTON_MAXIT;
+  uint64_t mneg[NM];
+  {
+    double m[NM];
+    targets(ubx, uby, T, m);
+    mneg[0] = 1ull << 63;
+#pragma unroll
+    for (int k = 1; k < NM; ++k) mneg[k] = 0u - fix_of_f64(m[k]);
+  }
+  float dl[NM];
+  float bound = INFINITY;  // of the last step's exponent changes
+  for (int r = 0;; ++r) {
+    float g32[NM];
+    if (bound <= FIX_STEP_MAX) {
+      PassMulFix pu(col, stride, mneg, bound);
+      visit_speeds<float>(dl, pu, 0.0f);
+      ++*updates;
+#pragma unroll
+      for (int k = 0; k < NM; ++k) g32[k] = fix_residual_f32(pu.M[k]);
+    } else {
+      if (!(exponent_bound(lam) < FIX_S_MAX)) return NEWTON_MAXIT;
+      Oct mu[NM];
+      mu[0] = fixe::oct((uint32_t)__float2int_rn(mul_rn(1.0f + lam[0], FIX_SCALE)));
+#pragma unroll
+      for (int k = 1; k < NM; ++k) mu[k] = fixe::oct((uint32_t)__float2int_rn(mul_rn(lam[k], FIX_SCALE)));
+      PassFix ps(tab, col, stride, mneg);
+      visit_speeds<Oct>(mu, ps, Oct(0));
+      ++*evals;
+      if (ps.ymax >= FIX_Y_END) return NEWTON_MAXIT;
+#pragma unroll
+      for (int k = 0; k < NM; ++k) g32[k] = fix_residual_f32(ps.M[k]);
+    }
+    float gmax = 0.0f;
+#pragma unroll
+    for (int k = 0; k < NM; ++k) gmax = fmaxf(gmax, fabsf(g32[k]));
+    if (gmax <= tolf) return NEWTON_OK;
+    if (r >= maxr) return NEWTON_MAXIT;
+    solve32(fc, g32, dl);
+    bound = step_exponent_bound(dl);  // (a NaN fails both comparisons)
+#pragma unroll
+    for (int k = 0; k < NM; ++k) lam[k] += dl[k];
+  }
+}
+
+// FP32 Newton from the warm start if given, else (or if that fails) from the
+// Maxwellian, then the fixed-point refinement: on NEWTON_OK the Q63 column and
+// the multipliers in lam.
+//
+// lam holds the warm start on entry if `warm` is set. Inlined: a call would save
+// and restore some sixty registers per thread through local memory, which
+// at two blocks of columns per SM leaves L1.
+__device__ __forceinline__ int solve_fix(double ubx, double uby, double T, float tolf, bool warm,
+                                         const uint64_t* ftab, uint64_t* col, int stride,
+                                         float lam[NM], SolveCount* cnt) {
+  const float ubx32 = cvt_f32_rn(ubx), uby32 = cvt_f32_rn(uby), T32 = cvt_f32_rn(T);
+  Fact32 fc;
+  float gres = 0.0f;
+  int st;
+  for (bool w = warm;; w = false) {
+    int it32 = 0;
+    st = newton_fp32(ubx32, uby32, T32, 30, w, lam, fc, &it32, &gres);
+    cnt->fp32_iters += it32;
+    if (st == NEWTON_OK || !w) break;
+  }
+  if (st == NEWTON_OK) {
+    int ev = 0, up = 0;
+    st = refine_fix(ubx, uby, T, tolf, 6, lam, fc, gres, ftab, col, stride, &ev, &up);
+    cnt->fp64_evals += ev;
+    cnt->fp64_updates += up;
+  }
+  return st;
+}
+
+// Equilibrium of the FP32 form by FP32 Newton (from the warm start if given,
+// else from the Maxwellian; again from the Maxwellian if the warm start fails),
+// FP64 refinement, full FP64 Newton as the last fallback. The FP64 equilibrium
+// per unit density lands in col[i * stride]; the multipliers in lam32 (FP32, as
+// the warm start keeps them) and, if lam64 is given, in FP64. It serves the
+// states solve_fix does not take and the callers that want FP64 multipliers.
+static __device__ __noinline__ int equilibrium_mixed(double ubx, double uby, double T, double tol,
+                                                     int maxit, const double* tab,
+                                                     const float* warm, double* col, int stride,
+                                                     float lam32[NM], double* lam64,
+                                                     SolveCount* cnt) {
   if (!(T > 0.0) || !isfinite(T) || !isfinite(ubx) || !isfinite(uby)) return NEWTON_UNREALIZABLE;
   float l32[NM];
   Fact32 fc;
-  int it32 = 0, ev = 0;
+  float gres = 0.0f;
+  int ev = 0;
   int st = NEWTON_SINGULAR;
   const float ubx32 = cvt_f32_rn(ubx), uby32 = cvt_f32_rn(uby), T32 = cvt_f32_rn(T);
-  if (warm) {
+  bool w = warm != nullptr;
+  if (w)
 #pragma unroll
     for (int k = 0; k < NM; ++k) l32[k] = warm[k];
-    st = newton_fp32(ubx32, uby32, T32, 30, true, l32, fc, &it32);
+  for (;;) {
+    int it32 = 0;
+    st = newton_fp32(ubx32, uby32, T32, 30, w, l32, fc, &it32, &gres);
     cnt->fp32_iters += it32;
-  }
-  if (st != NEWTON_OK) {
-    st = newton_fp32(ubx32, uby32, T32, 30, false, l32, fc, &it32);
-    cnt->fp32_iters += it32;
+    if (st == NEWTON_OK || !w) break;
+    w = false;
   }
   if (st == NEWTON_OK) {
     int up = 0;

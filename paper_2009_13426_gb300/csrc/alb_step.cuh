@@ -2,9 +2,10 @@
 // single-flow and the batched kernels.
 //
 // One thread updates one node. Its pulled populations (42, precision P) and
-// the 21 FP64 equilibrium values per unit density of its latest equilibrium
-// solve sit in two columns of the block's dynamic shared memory, with the
-// block size as stride.
+// the 21 equilibrium values per unit density of its latest equilibrium solve
+// (64 bits each: FP64, or Q63 fixed point from the FP32 form's solver) sit in
+// two columns of the block's dynamic shared memory, with the block size as
+// stride.
 #pragma once
 
 #include <type_traits>
@@ -16,67 +17,109 @@ namespace alb {
 
 constexpr int BLOCK = 128;
 
+// Dynamic shared memory of a block: the fixed-point exponential's table (FP32
+// form), then the two columns of every thread.
+template <typename P>
+constexpr size_t table_bytes() {
+  return std::is_same<P, float>::value ? FIXT_N * sizeof(uint64_t) : 0;
+}
 template <typename P, int B = BLOCK>
 constexpr size_t smem_bytes() {
-  return (size_t)NPLANES * B * sizeof(P) + (size_t)Q * B * sizeof(double);
+  return table_bytes<P>() + (size_t)NPLANES * B * sizeof(P) + (size_t)Q * B * sizeof(double);
 }
 
 // Shared columns of this thread: populations (P) and equilibrium (double),
-// both with stride B (the block size).
+// both with stride B (the block size); the tables of the solves.
 template <typename P, int B>
 struct Columns {
   P* pop;
   double* eq;
-  __device__ __forceinline__ Columns(unsigned char* smem) {
-    pop = reinterpret_cast<P*>(smem) + threadIdx.x;
-    eq = reinterpret_cast<double*>(smem + (size_t)NPLANES * B * sizeof(P)) + threadIdx.x;
+  const uint64_t* fixtab;
+  const double* exptab;
+  // All threads of the block construct it (load_exptab includes a barrier);
+  // s_exptab: EXPT_N doubles of shared memory.
+  __device__ __forceinline__ Columns(unsigned char* smem, double* s_exptab) {
+    if constexpr (std::is_same<P, float>::value) load_fixtab(reinterpret_cast<uint64_t*>(smem));
+    load_exptab(s_exptab);
+    fixtab = reinterpret_cast<const uint64_t*>(smem);
+    exptab = s_exptab;
+    pop = reinterpret_cast<P*>(smem + table_bytes<P>()) + threadIdx.x;
+    eq = reinterpret_cast<double*>(smem + table_bytes<P>() + (size_t)NPLANES * B * sizeof(P)) +
+         threadIdx.x;
   }
 };
 
 // Equilibrium of one node in the storage precision P: the full FP64 Newton for
-// the FP64 plain path, the mixed FP32/FP64 solver for the FP32 form, both
-// started from `warm` (multipliers in precision P) when given. The
-// equilibrium per unit density lands in eq[i * B], the multipliers (in the
-// precision P the warm start keeps them in) in lam.
-template <typename P, int B = BLOCK>
-__device__ __forceinline__ int node_equilibrium(const Params& pr, double ubx, double uby,
-                                                double T, const double* tab, const P* warm,
-                                                double* eq, P lam[NM], SolveCount* cnt) {
+// the FP64 plain path, FP32 Newton with the fixed-point refinement for the FP32
+// form (FP64 refinement where that does not reach), both started from the
+// multipliers in lam (precision P) if `warm` is set. The equilibrium per unit
+// density lands in the thread's column (Q63 instead of FP64 where *fixed is
+// set), the multipliers (in the precision P the warm start keeps them in) in
+// lam; after a failure lam is the warm start again.
+template <typename P, int B>
+__device__ __forceinline__ int node_equilibrium(const Params& pr, const Columns<P, B>& cl,
+                                                double ubx, double uby, double T, bool warm,
+                                                P lam[NM], SolveCount* cnt, bool* fixed) {
+  *fixed = false;
+  if (!(T > 0.0) || !isfinite(T) || !isfinite(ubx) || !isfinite(uby)) return NEWTON_UNREALIZABLE;
+  P w[NM];
+#pragma unroll
+  for (int k = 0; k < NM; ++k) w[k] = lam[k];
+  int st;
   if (pr.moments == 4) {
     // reduced model: FP64 4x4 Newton in both precisions
     double w8[NM], l8[NM];
     if (warm)
 #pragma unroll
-      for (int k = 0; k < NM; ++k) w8[k] = (double)warm[k];
+      for (int k = 0; k < NM; ++k) w8[k] = (double)lam[k];
     int it = 0, ev = 0;
-    int st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, tab, eq, B, l8, &it, &ev,
-                           warm ? w8 : nullptr);
+    st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l8, &it, &ev,
+                       warm ? w8 : nullptr);
     cnt->fp64_iters += it;
     cnt->fp64_evals += ev;
     if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
-      st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, tab, eq, B, l8, &it, &ev, nullptr);
+      st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l8, &it, &ev, nullptr);
       cnt->fp64_iters += it;
       cnt->fp64_evals += ev;
     }
 #pragma unroll
     for (int k = 0; k < NM; ++k) lam[k] = (P)l8[k];
-    return st;
-  }
-  if constexpr (std::is_same<P, float>::value) {
-    return equilibrium_mixed(ubx, uby, T, pr.tol, pr.maxit, tab, warm, eq, B, lam, nullptr, cnt);
+  } else if constexpr (std::is_same<P, float>::value) {
+    st = solve_fix(ubx, uby, T, (float)pr.tol, warm, cl.fixtab, reinterpret_cast<uint64_t*>(cl.eq),
+                   B, lam, cnt);
+    *fixed = st == NEWTON_OK;
+    if (st != NEWTON_OK) {
+      SolveCount c;  // of its own: the callers' counts stay in registers
+      float l32[NM];
+#pragma unroll
+      for (int k = 0; k < NM; ++k) l32[k] = w[k];
+      st = equilibrium_mixed(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, warm ? l32 : nullptr, cl.eq,
+                             B, l32, nullptr, &c);
+      cnt->add(c);
+#pragma unroll
+      for (int k = 0; k < NM; ++k) lam[k] = l32[k];
+    }
   } else {
     int it = 0, ev = 0;
-    int st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, tab, eq, B, lam, &it, &ev, warm);
+    double l64[NM];
+    st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l64, &it, &ev,
+                      warm ? w : nullptr);
     cnt->fp64_iters += it;
     cnt->fp64_evals += ev;
     if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
       // the previous multipliers led nowhere: start again from the Maxwellian
-      st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, tab, eq, B, lam, &it, &ev, nullptr);
+      st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l64, &it, &ev, nullptr);
       cnt->fp64_iters += it;
       cnt->fp64_evals += ev;
     }
-    return st;
+#pragma unroll
+    for (int k = 0; k < NM; ++k) lam[k] = l64[k];
   }
+  if (st != NEWTON_OK) {
+#pragma unroll
+    for (int k = 0; k < NM; ++k) lam[k] = w[k];
+  }
+  return st;
 }
 
 // Moment accumulation: plain in FP64; Neumaier-compensated in FP32.
@@ -84,6 +127,7 @@ template <typename P>
 struct Acc {
   double s = 0.0;
   __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void add_times(double v, int w) { s = fma(v, (double)w, s); }
   __device__ __forceinline__ double val() const { return s; }
 };
 template <>
@@ -97,8 +141,13 @@ struct Acc<float> {
       c += (v - t) + s;
     s = t;
   }
+  // w v with the product's rounding error kept (products by 3 and 9 round)
+  __device__ __forceinline__ void add_times(float v, int w) {
+    const float p = mul_rn(v, (float)w);
+    if (w & (w - 1)) c += fmaf(v, (float)w, -p);
+    add(p);
+  }
   __device__ __forceinline__ double val() const { return cvt_f64(s + c); }
-  __device__ __forceinline__ float valf() const { return s + c; }
 };
 
 // Multipliers stored for node k (8 planes of L), moved into the frame of
@@ -118,24 +167,28 @@ __device__ __forceinline__ void load_warm(const L* lam, size_t ps, size_t k, int
   }
 }
 
+// One value of an equilibrium column in FP64.
+template <typename P>
+__device__ __forceinline__ double eq_f64(double v, bool fixed) {
+  if constexpr (std::is_same<P, float>::value) {
+    if (fixed) return fix_to_f64((uint64_t)__double_as_longlong(v));
+  }
+  return v;
+}
+
 // Grad rebuild of a missing pull (Sec. III.B.2, IV.A.3): the post-collision
 // population of velocity i = (cx, cy) in the receiver's lattice (Upx, Upy),
 // built from the sender's moments at (sx, sy) (possibly a ghost), their
 // central differences and the sender's relaxation time:
 // h* = h^eq (1 + (1 - 1/tau) phi_h), plus (1/tau - 1/tau_Pr) h^eq phi_h,q for
-// Pr != 1 (the collision of App. E applied to the Grad population). Uses the
-// thread's equilibrium column as scratch. Returns 1 if the root finder failed
-// and the Maxwellian-guess fallback was used. With eq_led given, the
-// equilibrium of this sender in this lattice has been solved already (by
-// another pull of the block): its column eq_led and whether that solve
-// failed (led_failed) take the place of the solve.
-template <typename P, int B>
-__device__ __noinline__ int rebuild_pull(const Params pr, const P* __restrict__ mom, size_t ps,
-                                         int i, int cx, int cy, int Upx, int Upy, int sx, int sy,
-                                         double* fi, double* gi, const double* tab, double* eq,
-                                         const P* lam_in, const uint8_t* lat_in,
-                                         SolveCount* cnt, const double* eq_led = nullptr,
-                                         int led_failed = 0) {
+// Pr != 1 (the collision of App. E applied to the Grad population). `eq` is the
+// equilibrium per unit density of velocity i from the solve of this sender in
+// this lattice; ok is false if that solve failed: then the value of the
+// Maxwellian guess is taken.
+template <typename P>
+__device__ __forceinline__ void rebuild_value(const Params& pr, const P* __restrict__ mom,
+                                              size_t ps, int cx, int cy, int Upx, int Upy, int sx,
+                                              int sy, double eq, bool ok, double* fi, double* gi) {
   bool gh = false;
   const int rx = resolve(sx, pr.nx, pr.bcx, &gh);
   const int ry = resolve(sy, pr.ny, pr.bcy, &gh);
@@ -146,77 +199,66 @@ __device__ __noinline__ int rebuild_pull(const Params pr, const P* __restrict__ 
   const size_t nx = (size_t)pr.nx;
   const size_t ks = ry * nx + rx;
   const size_t kxp = ry * nx + xp, kxm = ry * nx + xm, kyp = yp * nx + rx, kym = ym * nx + rx;
-  const P* mr = mom;
   const P* mux = mom + ps;
   const P* muy = mom + 2 * ps;
   const P* mT = mom + 3 * ps;
-  const double rho = (double)mr[ks], ux = (double)mux[ks], uy = (double)muy[ks],
+  const double rho = (double)mom[ks], ux = (double)mux[ks], uy = (double)muy[ks],
                T = (double)mT[ks];
-  double du[2][2], dT[2];
-  du[0][0] = 0.5 * ((double)mux[kxp] - (double)mux[kxm]);
-  du[1][0] = 0.5 * ((double)mux[kyp] - (double)mux[kym]);
-  du[0][1] = 0.5 * ((double)muy[kxp] - (double)muy[kxm]);
-  du[1][1] = 0.5 * ((double)muy[kyp] - (double)muy[kym]);
-  dT[0] = 0.5 * ((double)mT[kxp] - (double)mT[kxm]);
-  dT[1] = 0.5 * ((double)mT[kyp] - (double)mT[kym]);
-  const double ubx = ux - Upx, uby = uy - Upy;
-  int st;
-  if (eq_led) {
-    st = led_failed ? NEWTON_MAXIT : NEWTON_OK;
-    eq = const_cast<double*>(eq_led);  // read only below
-  } else {
-    P lam[NM];
-    P wbuf[NM];
-    const P* warm = nullptr;
-    if (pr.warm) {
-      load_warm<P>(lam_in, ps, ks, lat_in[ks], Upx, Upy, wbuf);
-      warm = wbuf;
-    }
-    st = (rho > 0.0) ? node_equilibrium<P, B>(pr, ubx, uby, T, tab, warm, eq, lam, cnt)
-                     : NEWTON_UNREALIZABLE;
-  }
-  const double gfac = (2.0 * pr.cv - 2.0) * T;
-  if (st != NEWTON_OK) {
+  const double gfac = mul_rn(fma(2.0, pr.cv, -2.0), T);
+  if (!ok) {
     if (T > 0.0) {
       double lam[NM];
-      maxwellian_guess(ubx, uby, T, lam);
-      *fi = rho * exp_family_one(lam, cx, cy);
+      maxwellian_guess(ux - Upx, uy - Upy, T, lam);
+      *fi = mul_rn(rho, exp_family_one(lam, cx, cy));
     } else {
       *fi = 0.0;
     }
-    *gi = gfac * (*fi);
-    return 1;
+    *gi = mul_rn(gfac, *fi);
+    return;
   }
+  double du[2][2], dT[2];
+  du[0][0] = mul_rn(0.5, (double)mux[kxp] - (double)mux[kxm]);
+  du[1][0] = mul_rn(0.5, (double)mux[kyp] - (double)mux[kym]);
+  du[0][1] = mul_rn(0.5, (double)muy[kxp] - (double)muy[kxm]);
+  du[1][1] = mul_rn(0.5, (double)muy[kyp] - (double)muy[kym]);
+  dT[0] = mul_rn(0.5, (double)mT[kxp] - (double)mT[kxm]);
+  dT[1] = mul_rn(0.5, (double)mT[kyp] - (double)mT[kym]);
   const double tau = 0.5 + pr.nu / T;
   const double omega = 1.0 - 1.0 / tau;
-  const double feq = rho * eq[i * B];
+  const double feq = mul_rn(rho, eq);
   const double cbx = (double)(cx + Upx) - ux;
   const double cby = (double)(cy + Upy) - uy;
   double phf, phg, phq;
   grad_phi(pr, rho, T, cbx, cby, du, dT, &phf, &phg, &phq);
+  double ff = fma(omega, phf, 1.0), fg = fma(omega, phg, 1.0);
   if (pr.shakhov) {
-    const double w = 1.0 / tau - 1.0 / (0.5 + (pr.nu / pr.prandtl) / T);
-    *fi = feq * (1.0 + omega * phf + w * phq);
-    *gi = gfac * feq * (1.0 + omega * phg + w * phg);
-  } else {
-    *fi = feq * (1.0 + omega * phf);
-    *gi = gfac * feq * (1.0 + omega * phg);
+    const double w = 1.0 / tau - 1.0 / (0.5 + pr.kappa_nu / T);
+    ff = fma(w, phq, ff);
+    fg = fma(w, phg, fg);
   }
-  return 0;
+  *fi = mul_rn(feq, ff);
+  *gi = mul_rn(mul_rn(gfac, feq), fg);
 }
 
-// The equilibrium column (FP64 values per unit density at stride B) in the
+// The equilibrium column (values per unit density at stride B) in the
 // population precision. In the FP32 form every value is rounded to FP32 once,
-// in place, into the first word of its slot (the FP64 value is not read
+// in place, into the first word of its slot (the 64-bit value is not read
 // again), so that the sensor, the BGK update and the App. E term read the
-// same float; the rounding runs on the integer pipe (cvt_f32_rn), not the
-// FP64 pipe. Element i is then at [i * eq_stride<P, B>()].
+// same float; the rounding runs on the integer pipe (fix_to_f32, or cvt_f32_rn
+// of a column in FP64), not the FP64 pipe. Element i is then at
+// [i * eq_stride<P, B>()].
 template <typename P, int B>
-__device__ __forceinline__ const P* eq_in_precision(double* eq) {
+__device__ __forceinline__ const P* eq_in_precision(double* eq, bool fixed) {
   if constexpr (std::is_same<P, float>::value) {
     float* v = reinterpret_cast<float*>(eq);
+    if (fixed) {
 #pragma unroll
-    for (int i = 0; i < Q; ++i) v[2 * i * B] = cvt_f32_rn(eq[i * B]);
+      for (int i = 0; i < Q; ++i)
+        v[2 * i * B] = fix_to_f32((uint64_t)__double_as_longlong(eq[i * B]));
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < Q; ++i) v[2 * i * B] = cvt_f32_rn(eq[i * B]);
+    }
     return v;
   } else {
     return eq;
@@ -251,47 +293,48 @@ __device__ __forceinline__ void store_shakhov(const Params& pr, const P* st, con
   const P Tp = (P)T, rp = (P)rho;
   const P bx = (P)(ux - (double)lat_ux(code)), by = (P)(uy - (double)lat_uy(code));
   const P cp = (P)pr.cp;
-  const P gp = ((P)2 * (P)pr.cv - (P)2) * Tp;
-  const P tau_pr = ((P)0.5 + (P)(pr.nu / pr.prandtl) / Tp) * (tau / ((P)0.5 + (P)pr.nu / Tp));
+  const P gp = mul_rn(fma((P)2, (P)pr.cv, (P)-2), Tp);
+  const P tau_pr = mul_rn((P)0.5 + (P)pr.kappa_nu / Tp, tau / ((P)0.5 + (P)pr.nu / Tp));
   const P om = (P)1 / tau;
   const P w = om - (P)1 / tau_pr;
   P qx = 0, qy = 0;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
     const P cx = (P)XI_X(i) - bx, cy = (P)XI_Y(i) - by;
-    const P e = (cx * cx + cy * cy) * st[i * B] + st[(Q + i) * B];
-    qx += cx * e;
-    qy += cy * e;
+    const P e = fma(fma(cx, cx, mul_rn(cy, cy)), st[i * B], st[(Q + i) * B]);
+    qx = fma(cx, e, qx);
+    qy = fma(cy, e, qy);
   }
-  qx *= (P)0.5;
-  qy *= (P)0.5;
-  const P af = w / (rp * cp * Tp * Tp);
-  const P ag = w * (P)2 / (rp * cp);
+  qx = mul_rn(qx, (P)0.5);
+  qy = mul_rn(qy, (P)0.5);
+  const P rc = mul_rn(rp, cp);
+  const P af = w / mul_rn(mul_rn(rc, Tp), Tp);
+  const P ag = mul_rn(w, (P)2) / rc;
   const P h = (P)0.5 / Tp;
 #pragma unroll
   for (int i = 0; i < Q; ++i) {
-    const P fe = eqv[i * eq_stride<P, B>()] * rp;
-    const P ge = gp * fe;
+    const P fe = mul_rn(eqv[i * eq_stride<P, B>()], rp);
+    const P ge = mul_rn(gp, fe);
     const P f = st[i * B];
     const P g = st[(Q + i) * B];
     const P cx = (P)XI_X(i) - bx, cy = (P)XI_Y(i) - by;
-    const P c2 = cx * cx + cy * cy;
-    const P qc = qx * cx + qy * cy;
-    __stcs(&pop_out[i * ps + k], fma(om, fe - f, f) + af * qc * (c2 * h - cp) * fe);
-    __stcs(&pop_out[(Q + i) * ps + k], fma(om, ge - g, g) + ag * qc * ge);
+    const P c2 = fma(cx, cx, mul_rn(cy, cy));
+    const P qc = fma(qx, cx, mul_rn(qy, cy));
+    __stcs(&pop_out[i * ps + k],
+           fma(mul_rn(mul_rn(af, qc), fma(c2, h, -cp)), fe, fma(om, fe - f, f)));
+    __stcs(&pop_out[(Q + i) * ps + k], fma(mul_rn(ag, qc), ge, fma(om, ge - g, g)));
   }
 }
 
-// Moments, next shift, equilibrium and BGK of one node whose 42 pre-collision
-// populations sit in its shared column, then store.
+// Moments of one node whose 42 pre-collision populations sit in its shared
+// column, and the lattice of its next pull.
+struct NodeState {
+  double rho, ubx, uby, T;  // density, velocity in the lattice frame, temperature
+  int code2;                // next lattice
+};
 template <typename P, int B>
-__device__ __forceinline__ void collide_store(const Params& pr, const Columns<P, B>& cl, int code,
-                                              size_t k, size_t ps, P* __restrict__ pop_out,
-                                              P* __restrict__ mom_out, uint8_t* lat_out,
-                                              uint8_t* nxt_out, const double* tab,
-                                              const P* warm, P* lam_out,
-                                              SolveCount* cnt, unsigned* n_fail,
-                                              const uint8_t* nb = nullptr) {
+__device__ __forceinline__ NodeState node_moments(const Params& pr, const Columns<P, B>& cl,
+                                                  int code, const uint8_t* nb) {
   const P* st = cl.pop;
   const int Ux = lat_ux(code), Uy = lat_uy(code);
   Acc<P> ar, ajx, ajy, ae;
@@ -300,10 +343,10 @@ __device__ __forceinline__ void collide_store(const Params& pr, const Columns<P,
     const P f = st[i * B];
     const P g = st[(Q + i) * B];
     ar.add(f);
-    if (XI_X(i) != 0) ajx.add(XI_X(i) == 1 ? f : XI_X(i) == -1 ? -f : (P)XI_X(i) * f);
-    if (XI_Y(i) != 0) ajy.add(XI_Y(i) == 1 ? f : XI_Y(i) == -1 ? -f : (P)XI_Y(i) * f);
+    if (XI_X(i) != 0) ajx.add_times(XI_X(i) > 0 ? f : -f, abs(XI_X(i)));
+    if (XI_Y(i) != 0) ajy.add_times(XI_Y(i) > 0 ? f : -f, abs(XI_Y(i)));
     const int c2 = XI_X(i) * XI_X(i) + XI_Y(i) * XI_Y(i);
-    if (c2 != 0) ae.add(c2 == 1 ? f : (P)c2 * f);
+    if (c2 != 0) ae.add_times(f, c2);
     ae.add(g);
   }
   // Moments (Eq. polyTemp). The velocity and temperature that define the
@@ -316,13 +359,13 @@ __device__ __forceinline__ void collide_store(const Params& pr, const Columns<P,
     // FP32 sums: one FP64 reciprocal serves the three quotients (their last
     // FP64 bit lies far below the sums' own precision); 1/(2 Cv) = (gamma-1)/2
     const double ir = 1.0 / rho;
-    ubx = ajx.val() * ir;
-    uby = ajy.val() * ir;
-    T = (ae.val() - rho * (ubx * ubx + uby * uby)) * ir * pr.half_gm1;
+    ubx = mul_rn(ajx.val(), ir);
+    uby = mul_rn(ajy.val(), ir);
+    T = mul_rn(mul_rn(fma(-rho, fma(ubx, ubx, mul_rn(uby, uby)), ae.val()), ir), pr.half_gm1);
   } else {
     ubx = ajx.val() / rho;
     uby = ajy.val() / rho;
-    T = (ae.val() - rho * (ubx * ubx + uby * uby)) / (2.0 * rho * pr.cv);
+    T = fma(-rho, fma(ubx, ubx, mul_rn(uby, uby)), ae.val()) / mul_rn(2.0 * rho, pr.cv);
   }
   const double ux = ubx + cvt_f64(Ux), uy = uby + cvt_f64(Uy);
   // next lattice: Eq. criterion, or overlapping ranges chosen by history or
@@ -331,41 +374,47 @@ __device__ __forceinline__ void collide_store(const Params& pr, const Columns<P,
   const int code2 = by_nb ? lat_code(select_shift_neighbours(ux, 0, nb, pr),
                                      select_shift_neighbours(uy, 1, nb, pr))
                           : lat_code(select_shift_kept(ux, Ux, pr), select_shift_kept(uy, Uy, pr));
+  return NodeState{rho, ubx, uby, T, code2};
+}
 
-  P lam[NM];
-  const int ns = (rho > 0.0) ? node_equilibrium<P, B>(pr, ubx, uby, T, tab, warm, cl.eq, lam, cnt)
-                             : NEWTON_UNREALIZABLE;
+// Collision of a node (BGK, or App. E for Pr != 1) with the equilibrium in its
+// column (solve status ns, multipliers lam: the warm start's after a failure),
+// then the store of its state. A failed node is left uncollided and counted.
+template <typename P, int B>
+__device__ __forceinline__ void node_store(const Params& pr, const Columns<P, B>& cl, int code,
+                                           const NodeState& s, int ns, bool fixed, bool warm,
+                                           const P lam[NM], size_t k, size_t ps,
+                                           P* __restrict__ pop_out, P* __restrict__ mom_out,
+                                           uint8_t* lat_out, uint8_t* nxt_out, P* lam_out,
+                                           unsigned* n_fail) {
+  const P* st = cl.pop;
+  const double rho = s.rho, T = s.T;
+  const double ux = s.ubx + cvt_f64(lat_ux(code)), uy = s.uby + cvt_f64(lat_uy(code));
   // multipliers for the next step's warm start (lattice `code`), if stored
   if (lam_out) {
-    if (ns == NEWTON_OK) {
 #pragma unroll
-      for (int j = 0; j < NM; ++j) lam_out[j * ps + k] = lam[j];
-    } else if (warm) {
-#pragma unroll
-      for (int j = 0; j < NM; ++j) lam_out[j * ps + k] = warm[j];
-    } else {
-#pragma unroll
-      for (int j = 0; j < NM; ++j) lam_out[j * ps + k] = j == 3 || j == 5 ? (P)0.5 : (P)0;
-    }
+    for (int j = 0; j < NM; ++j)
+      lam_out[j * ps + k] =
+          ns == NEWTON_OK || warm ? lam[j] : (j == 3 || j == 5 ? (P)0.5 : (P)0);
   }
   if (ns == NEWTON_OK) {
     // f^eq = rho p, g^eq = (2 Cv - D) T f^eq and tau = 1/2 + nu/T in the
     // population precision (in the FP32 form from the FP64 equilibrium)
     const P Tp = to_p<P>(T);
-    const P gp = ((P)2 * to_p<P>(pr.cv) - (P)2) * Tp;
+    const P gp = mul_rn(fma((P)2, to_p<P>(pr.cv), (P)-2), Tp);
     P tau = (P)0.5 + to_p<P>(pr.nu) / Tp;
     const P rp = to_p<P>(rho);
-    const P* eqv = eq_in_precision<P, B>(cl.eq);
+    const P* eqv = eq_in_precision<P, B>(cl.eq, fixed);
     constexpr int es = eq_stride<P, B>();
     if (pr.sensor) {
       P eps = 0;
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        const P fe = eqv[i * es] * rp;
+        const P fe = mul_rn(eqv[i * es], rp);
         eps += rel_dev(st[i * B], fe);
       }
       eps /= (P)Q;
-      tau *= sensor_alpha<P>(pr, eps);
+      tau = mul_rn(tau, sensor_alpha<P>(pr, eps));
     }
     if (pr.shakhov) {
       store_shakhov<P, B>(pr, st, eqv, rho, ux, uy, T, code, tau, k, ps, pop_out);
@@ -373,8 +422,8 @@ __device__ __forceinline__ void collide_store(const Params& pr, const Columns<P,
       const P om = (P)1 / tau;
 #pragma unroll
       for (int i = 0; i < Q; ++i) {
-        const P fe = eqv[i * es] * rp;
-        const P ge = gp * fe;
+        const P fe = mul_rn(eqv[i * es], rp);
+        const P ge = mul_rn(gp, fe);
         const P f = st[i * B];
         const P g = st[(Q + i) * B];
         __stcs(&pop_out[i * ps + k], fma(om, fe - f, f));
@@ -391,7 +440,7 @@ __device__ __forceinline__ void collide_store(const Params& pr, const Columns<P,
   mom_out[2 * ps + k] = to_p<P>(uy);
   mom_out[3 * ps + k] = to_p<P>(T);
   lat_out[k] = (uint8_t)code;
-  nxt_out[k] = (uint8_t)code2;
+  nxt_out[k] = (uint8_t)s.code2;
 }
 
 // Current lattices of the eight nodes around (x, y) (boundary rule for
@@ -428,32 +477,111 @@ __device__ __forceinline__ void flush_counts(unsigned long long* ctr, const Node
   warp_count(ctr + CTR_REC_FAIL, c.rec_fail);
 }
 
-// Shared state of a block's rebuild queue: one entry (owner thread << 5 | i)
-// per missing pull of the block's nodes, at most Q per node.
+// Shared state of a block's rebuilds: one entry (owner thread << 5 | i) per
+// missing pull of the block's nodes, at most Q per node. They are handled in
+// chunks of CHUNK entries; within a chunk, every distinct (sender, receiver
+// lattice) is entered once into a hash table and solved once.
 template <int B>
 struct RebuildQueue {
+  static constexpr int PER = 3;          // entries per thread and chunk
+  static constexpr int CHUNK = PER * B;
+  static constexpr int HASH = 4 * B;     // positions (a power of two), at most 3/4 used
+  static constexpr int SHIFT = B == 32 ? 25 : B == 64 ? 24 : B == 128 ? 23 : 22;  // 32 - log2(HASH)
+  static_assert(HASH == 1 << (32 - SHIFT), "hash positions");
   unsigned short entry[Q * B];
-  unsigned key[B];             // (receiver lattice, sender position in the tile's frame)
-  unsigned char failed[B];     // the entry's own solve fell back
-  unsigned short slot[B];      // leader entry solved by thread j
-  unsigned short solver[B];    // thread solving a leader entry
-  int wsum[B / 32];            // missing pulls per warp
-  int count;
+  unsigned hkey[HASH];          // key of a position, or EMPTY
+  unsigned short hslot[HASH];   // its solve
+  unsigned skey[CHUNK];         // key of each solve
+  unsigned char state[B];       // of the solves of a round: 1 failed, 2 column in Q63
+  int wsum[B / 32];             // missing pulls per warp
+  int count, nsolve;
 };
+constexpr unsigned RB_EMPTY = 0xffffffffu;
+
+// Key of a rebuild solve: receiver lattice and sender position in the tile's
+// frame. The sender lies within 6 nodes of the tile (|xi| <= 3, |U| <= 3) and
+// the tile's sides are at most B <= 1000: 10 bits per coordinate.
+__device__ __forceinline__ unsigned rebuild_key(int code, int sx, int sy) {
+  return ((unsigned)code << 20) | ((unsigned)(sy + 8) << 10) | (unsigned)(sx + 8);
+}
+
+// Asynchronous copy of one population from global into shared memory, evicted
+// first from L2 (populations are read once and written once per step; L2 is
+// kept for the lattice codes and the threads' stack).
+template <typename P>
+__device__ __forceinline__ void copy_async(P* dst, const P* src, unsigned long long policy) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global.L2::cache_hint [%0], [%1], %2, %3;" ::"r"(d), "l"(src),
+               "n"(sizeof(P)), "l"(policy)
+               : "memory");
+}
+__device__ __forceinline__ void async_copies_wait() {
+  asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+static __constant__ signed char c_xi[Q][2] = {
+    {0, 0},  {1, 0},   {0, 1},   {-1, 0}, {0, -1}, {1, 1},  {-1, 1}, {-1, -1}, {1, -1}, {2, 0}, {0, 2},
+    {-2, 0}, {0, -2},  {2, 2},   {-2, 2}, {-2, -2}, {2, -2}, {3, 0},  {0, 3},   {-3, 0}, {0, -3}};
+
+// Starts the pulls of node (x, y) in its lattice (Upx, Upy): the 42 populations
+// of its senders are copied into its shared-memory column by asynchronous
+// copies (all in flight together, without the 42 registers that loads would
+// hold), whether or not a sender turns out to live in this lattice. Returns the
+// mask of those that do; the others' entries are overwritten by their rebuilds.
+// Inside the grid the addresses are a common base plus one uniform offset per
+// velocity; at the grid's edges a rolled loop resolves each coordinate (an
+// index is inside the grid even for a ghost: resolve clamps it).
+template <typename P, int B>
+__device__ __forceinline__ unsigned pull_node(const StepArgs<P>& a, const Columns<P, B>& cl, int x,
+                                              int y, int code, int Upx, int Upy, bool inside) {
+  const Params& pr = a.prm;
+  const size_t ps = a.ps;
+  unsigned long long policy;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(policy));
+  unsigned own = 0;
+  if (inside) {
+    const size_t ks = (size_t)(y - Upy) * pr.nx + (x - Upx);
+    const P* src = a.pop_in + ks;
+    const uint8_t* lat = a.lat_in + ks;
+    int sc[Q];
+#pragma unroll
+    for (int i = 0; i < Q; ++i) {
+      const ptrdiff_t off = -((ptrdiff_t)XI_Y(i) * pr.nx + XI_X(i));
+      sc[i] = lat[off];
+      copy_async(cl.pop + i * B, src + (off + (ptrdiff_t)(i * ps)), policy);
+      copy_async(cl.pop + (Q + i) * B, src + (off + (ptrdiff_t)((Q + i) * ps)), policy);
+    }
+#pragma unroll
+    for (int i = 0; i < Q; ++i) own |= (sc[i] == code ? 1u : 0u) << i;
+  } else {
+#pragma unroll 1
+    for (int i = 0; i < Q; ++i) {
+      bool gh = false;
+      const int rx = resolve(x - c_xi[i][0] - Upx, pr.nx, pr.bcx, &gh);
+      const int ry = resolve(y - c_xi[i][1] - Upy, pr.ny, pr.bcy, &gh);
+      const size_t ks = (size_t)ry * pr.nx + rx;
+      copy_async(cl.pop + i * B, a.pop_in + (i * ps + ks), policy);
+      copy_async(cl.pop + (Q + i) * B, a.pop_in + ((Q + i) * ps + ks), policy);
+      // a ghost sender is always rebuilt
+      if (!gh && a.lat_in[ks] == code) own |= 1u << i;
+    }
+  }
+  return own;
+}
 
 // One time step of the nodes of a tile (Sec. IV.A.3), one node per thread:
 // thread t updates node (x0 + (t & (2^lg - 1)), y0 + (t >> lg)) if it lies in
 // the grid. Phase 1 pulls every population whose sender lives in the node's
 // new lattice and queues the missing ones; phase 2 rebuilds the queued pulls
-// with all threads of the block (each Grad rebuild is a full equilibrium
+// with all threads of the block (each distinct sender is a full equilibrium
 // solve, so spreading them keeps the warps of interface nodes from waiting on
 // a few lanes); phase 3 collides and stores. A rebuilt value depends only on
 // its inputs, not on the thread that computes it. All threads of the block
 // must call this (it holds barriers).
 template <typename P, int B>
 __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, int lg,
-                                          const Columns<P, B>& cl, const double* s_tab,
-                                          RebuildQueue<B>& rq, NodeCount& nc) {
+                                          const Columns<P, B>& cl, RebuildQueue<B>& rq,
+                                          NodeCount& nc) {
   const Params& pr = a.prm;
   const size_t ps = a.ps;
   const int t = threadIdx.x;
@@ -463,42 +591,15 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
   size_t k = 0;
   int code = 0;
   unsigned own = 0;  // bit i: the sender of velocity i lives in lattice `code`
+  // all senders of the tile lie in the grid (|xi| <= 3 and |U| <= 3)
+  const bool inside = x0 >= 6 && x0 + mask + 6 < pr.nx && y0 >= 6 && y0 + (B >> lg) + 5 < pr.ny;
   if (active) {
     k = (size_t)y * pr.nx + x;
     code = a.nxt_in[k];
     const int Upx = lat_ux(code), Upy = lat_uy(code);
-    // All loads first, so that they are in flight together (a pull's load
-    // written straight to shared memory would wait for the previous
-    // velocity's): for every velocity the sender's lattice code and its two
-    // populations, whether or not the sender turns out to live in this node's
-    // lattice (the index is inside the grid even for a ghost: resolve clamps
-    // it). Then the populations of the senders in this lattice go to the
-    // shared-memory column; the others are dropped and queued for a rebuild.
-    // Populations are read once and written once per step: streaming
-    // (evict-first) loads and stores keep L2 for the lattice codes and the
-    // threads' stack.
-    int sc[Q];
-    P v[2 * Q];
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      bool gh = false;
-      const int rx = resolve(x - XI_X(i) - Upx, pr.nx, pr.bcx, &gh);
-      const int ry = resolve(y - XI_Y(i) - Upy, pr.ny, pr.bcy, &gh);
-      const size_t ks = (size_t)ry * pr.nx + rx;
-      sc[i] = gh ? -1 : (int)a.lat_in[ks];  // a ghost sender is always rebuilt
-      v[i] = __ldcs(&a.pop_in[i * ps + ks]);
-      v[Q + i] = __ldcs(&a.pop_in[(Q + i) * ps + ks]);
-    }
-#pragma unroll
-    for (int i = 0; i < Q; ++i) own |= (sc[i] == code ? 1u : 0u) << i;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      if (own & (1u << i)) {
-        cl.pop[i * B] = v[i];
-        cl.pop[(Q + i) * B] = v[Q + i];
-      }
-    }
+    own = pull_node<P, B>(a, cl, x, y, code, Upx, Upy, inside);
   }
+  async_copies_wait();
   // The queue of missing pulls in (thread, velocity) order, placed by a
   // block-wide prefix sum of the threads' counts, so that its order, and with
   // it which pulls share a solve below, does not depend on scheduling. A tile
@@ -524,106 +625,124 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
       nq = rq.count;
     }
   }
-  P* pop0 = cl.pop - t;  // column 0 of the block
-  // Entries in chunks of B. The pulls of one sender in one receiver lattice
-  // need the same equilibrium (the sender's state in that lattice, from the
-  // same warm start). Within a chunk, the first entry of each such group (its
-  // leader) is solved, by threads 0, 1, ... in entry order, so that the solves
-  // fill as few warps as possible; every other entry then reads its leader's
-  // column after a barrier. A solve's result does not depend on the thread,
-  // so sharing it changes no value.
+  // Rebuild rounds, then the round of the node itself: the equilibrium solve is
+  // one inlined piece of code that both share. The distinct solves of a chunk
+  // run B at a time in the columns of threads 0, 1, ...; every entry then takes
+  // its value from the column of its solve (which entry comes first into the
+  // table, and which thread solves it, changes no value).
   static_assert(B % 32 == 0 && B <= 1000, "whole warps; tile sides fit the keys' 10-bit fields");
-  const int lane = t & 31, warp = t >> 5;
+  using RQ = RebuildQueue<B>;
+  P* const pop0 = cl.pop - t;  // column 0 of the block
+  int base = 0, round = 0, nsolve = 0;  // chunk, its solves done, its solves
+  unsigned short pos[RQ::PER];          // hash position of this thread's entries
 #pragma unroll 1
-  for (int base = 0; base < nq; base += B) {
-    const int ne = min(nq - base, B);
-    if (t < ne) {
-      const int owner = rq.entry[base + t] >> 5, i = rq.entry[base + t] & 31;
-      const int ox = x0 + (owner & mask), oy = y0 + (owner >> lg);
-      const int ocode = a.nxt_in[(size_t)oy * pr.nx + ox];
-      // the sender lies within 6 nodes of the tile (|xi| <= 3, |U| <= 3) and
-      // the tile's sides are at most B <= 1000: 10 bits per coordinate
-      const int sx = ox - XI_X(i) - lat_ux(ocode) - x0 + 8;
-      const int sy = oy - XI_Y(i) - lat_uy(ocode) - y0 + 8;
-      rq.key[t] = ((unsigned)ocode << 20) | ((unsigned)sy << 10) | (unsigned)sx;
-    }
-    __syncthreads();
-    int lead = -1;
-    if (t < ne) {
-      const unsigned key = rq.key[t];
-      lead = t;
-      for (int e = 0; e < t; ++e)
-        if (rq.key[e] == key) {
-          lead = e;
-          break;
-        }
-    }
-    // number the leaders (block-wide prefix sum of the leader flags)
-    const int isl = (t < ne && lead == t) ? 1 : 0;
-    int incl = isl;
+  for (;;) {
+    const bool rebuild = base < nq;
+    if (rebuild && round == 0) {
+      for (int j = t; j < RQ::HASH; j += B) rq.hkey[j] = RB_EMPTY;
+      if (t == 0) rq.nsolve = 0;
+      __syncthreads();
 #pragma unroll
-    for (int d = 1; d < 32; d <<= 1) {
-      const int u = __shfl_up_sync(0xffffffffu, incl, d);
-      if (lane >= d) incl += u;
-    }
-    if (lane == 31) rq.wsum[warp] = incl;
-    __syncthreads();
-    int nlead = 0, rank = incl - isl;
-    for (int w = 0; w < B / 32; ++w) {
-      nlead += rq.wsum[w];
-      if (w < warp) rank += rq.wsum[w];
-    }
-    if (isl) {
-      rq.slot[rank] = (unsigned short)t;    // solver thread rank -> leader entry
-      rq.solver[t] = (unsigned short)rank;  // leader entry -> its solver thread
-    }
-    __syncthreads();
-    // pass 0: thread j < nlead solves the j-th leader entry; pass 1: every
-    // other entry, with its leader's column
-#pragma unroll 1
-    for (int pass = 0; pass < 2; ++pass) {
-      if (pass) __syncthreads();
-      const int e = pass == 0 ? (t < nlead ? (int)rq.slot[t] : -1)
-                              : (t < ne && lead != t ? t : -1);
-      if (e >= 0) {
-        const int owner = rq.entry[base + e] >> 5, i = rq.entry[base + e] & 31;
-        const int ox = x0 + (owner & mask), oy = y0 + (owner >> lg);
-        const int ocode = a.nxt_in[(size_t)oy * pr.nx + ox];
-        const int Upx = lat_ux(ocode), Upy = lat_uy(ocode);
-        const int cx = XI_X(i), cy = XI_Y(i);
-        const int j = pass ? (int)rq.solver[lead] : t;  // thread whose column holds the solve
-        double fd, gd;
-        const int failed = rebuild_pull<P, B>(
-            pr, a.mom_in, ps, i, cx, cy, Upx, Upy, ox - cx - Upx, oy - cy - Upy, &fd, &gd, s_tab,
-            cl.eq, a.lam_in, a.lat_in, &nc.solve, pass ? cl.eq - t + j : nullptr,
-            pass ? rq.failed[lead] : 0);
-        if (!pass) {
-          rq.failed[e] = (unsigned char)failed;
-          nc.calls += 1;
+      for (int j = 0; j < RQ::PER; ++j) {
+        const int e = base + j * B + t;
+        pos[j] = 0;
+        if (e >= nq) continue;
+        const int owner = rq.entry[e] >> 5, i = rq.entry[e] & 31;
+        const int ox = owner & mask, oy = owner >> lg;
+        const int oc = a.nxt_in[(size_t)(y0 + oy) * pr.nx + (x0 + ox)];
+        const unsigned key =
+            rebuild_key(oc, ox - c_xi[i][0] - lat_ux(oc), oy - c_xi[i][1] - lat_uy(oc));
+        unsigned h = (key * 2654435761u) >> RQ::SHIFT;  // Knuth's multiplicative hash
+        for (;; h = (h + 1) % RQ::HASH) {
+          const unsigned old = atomicCAS(&rq.hkey[h], RB_EMPTY, key);
+          if (old == RB_EMPTY) {
+            const int slot = atomicAdd(&rq.nsolve, 1);
+            rq.hslot[h] = (unsigned short)slot;
+            rq.skey[slot] = key;
+            break;
+          }
+          if (old == key) break;
         }
-        nc.rec += 1;
-        nc.rec_fail += failed;
-        pop0[i * B + owner] = (P)fd;
-        pop0[(Q + i) * B + owner] = (P)gd;
+        pos[j] = (unsigned short)h;
       }
+      __syncthreads();
+      nsolve = rq.nsolve;
     }
-    // the next chunk reuses the columns, keys and slots; the last chunk's
-    // rebuilt pulls are in place before the collisions
+    // what to solve: the round's (sender, lattice) pairs, or the node
+    NodeState s;
+    s.rho = -1.0;
+    P lam[NM];
+    bool solve = false;
+    if (rebuild) {
+      if (round + t < nsolve) {
+        const unsigned key = rq.skey[round + t];
+        const int oc = key >> 20;
+        const int Upx = lat_ux(oc), Upy = lat_uy(oc);
+        bool gh = false;
+        const int rx = resolve(x0 + (int)(key & 1023u) - 8, pr.nx, pr.bcx, &gh);
+        const int ry = resolve(y0 + (int)((key >> 10) & 1023u) - 8, pr.ny, pr.bcy, &gh);
+        const size_t ks = (size_t)ry * pr.nx + rx;
+        s.rho = (double)a.mom_in[ks];
+        s.ubx = (double)a.mom_in[ps + ks] - Upx;
+        s.uby = (double)a.mom_in[2 * ps + ks] - Upy;
+        s.T = (double)a.mom_in[3 * ps + ks];
+        if (pr.warm) load_warm<P>(a.lam_in, ps, ks, a.lat_in[ks], Upx, Upy, lam);
+        solve = true;
+      }
+    } else if (active) {
+      uint8_t nb[8];
+      const bool by_nb = order_key(pr.overlap) > 0 && pr.rule == 1;
+      if (by_nb) neighbour_codes(pr, a.nxt_in, x, y, nb);
+      s = node_moments<P, B>(pr, cl, code, by_nb ? nb : nullptr);
+      if (pr.warm)
+        load_warm<P>(a.lam_in, ps, k, a.lat_in[k], lat_ux(code), lat_uy(code), lam);
+      solve = true;
+    }
+    int st = NEWTON_UNREALIZABLE;
+    bool fixed = false;
+    if (solve) {
+      nc.calls += 1;
+      if (s.rho > 0.0)
+        st = node_equilibrium<P, B>(pr, cl, s.ubx, s.uby, s.T, pr.warm, lam, &nc.solve, &fixed);
+    }
+    if (!rebuild) {
+      if (active)
+        node_store<P, B>(pr, cl, code, s, st, fixed, pr.warm, lam, k, ps, a.pop_out, a.mom_out,
+                         a.lat_out, a.nxt_out, a.lam_out, &nc.fail);
+      break;
+    }
+    rq.state[t] = (unsigned char)((st == NEWTON_OK ? 0 : 1) | (fixed ? 2 : 0));
     __syncthreads();
-  }
-  if (active) {
-    const int Upx = lat_ux(code), Upy = lat_uy(code);
-    P wbuf[NM];
-    const P* warm = nullptr;
-    if (pr.warm) {
-      load_warm<P>(a.lam_in, ps, k, a.lat_in[k], Upx, Upy, wbuf);
-      warm = wbuf;
+#pragma unroll 1
+    for (int j = 0; j < RQ::PER; ++j) {
+      const int e = base + j * B + t;
+      if (e >= nq) break;
+      const int j0 = (int)rq.hslot[j == 0 ? pos[0] : j == 1 ? pos[1] : pos[2]] - round;
+      if (j0 < 0 || j0 >= B) continue;  // solved in another round
+      const int owner = rq.entry[e] >> 5, i = rq.entry[e] & 31;
+      const int ox = x0 + (owner & mask), oy = y0 + (owner >> lg);
+      const int oc = a.nxt_in[(size_t)oy * pr.nx + ox];
+      const int Upx = lat_ux(oc), Upy = lat_uy(oc);
+      const int cx = c_xi[i][0], cy = c_xi[i][1];
+      const int state = rq.state[j0];
+      const bool ok = !(state & 1);
+      const double eq = ok ? eq_f64<P>(cl.eq[i * B - t + j0], state & 2) : 0.0;
+      double fd, gd;
+      rebuild_value<P>(pr, a.mom_in, ps, cx, cy, Upx, Upy, ox - cx - Upx, oy - cy - Upy, eq, ok,
+                       &fd, &gd);
+      nc.rec += 1;
+      nc.rec_fail += ok ? 0 : 1;
+      pop0[i * B + owner] = (P)fd;
+      pop0[(Q + i) * B + owner] = (P)gd;
     }
-    uint8_t nb[8];
-    if (order_key(pr.overlap) > 0 && pr.rule == 1) neighbour_codes(pr, a.nxt_in, x, y, nb);
-    collide_store<P, B>(pr, cl, code, k, ps, a.pop_out, a.mom_out, a.lat_out, a.nxt_out, s_tab,
-                        warm, a.lam_out, &nc.solve, &nc.fail, nb);
-    nc.calls += 1;
+    // the next round reuses the columns, the next chunk the table; after the
+    // last one the rebuilt pulls are in place before the collisions
+    __syncthreads();
+    round += B;
+    if (round >= nsolve) {
+      round = 0;
+      base += RQ::CHUNK;
+    }
   }
 }
 

@@ -14,6 +14,9 @@ accuracy uses the same table with the reduction r = x - n L in one step
 |x| < 700) and the Taylor polynomial of degree 3 (remainder below
 r^4/4! < 1.4e-13 on |r| <= ln2/512).
 
+The fixed-point exponential of the FP32 form (alb_fix.cuh) has a table of its
+own: 2^-(j/512), j = 0..511, rounded to 63 fraction bits.
+
 Every constant is computed here with 60-digit decimal arithmetic and rounded
 to the nearest double: T[j], N/ln2, the two-part split of ln2/N (high part
 with 33 significant bits so that n * high is exact for |n| < 2^20) and 1/k!.
@@ -56,6 +59,7 @@ BITS = 8
 N = 1 << BITS
 DEG = 4
 HI_BITS = 33
+FIXT_BITS = 9
 
 
 def main():
@@ -93,6 +97,18 @@ def main():
     for j in range(0, N, 2):
         tail = ", \\" if j < N - 2 else ""
         out.append("    %s, %s%s" % (hexd(table[j]), hexd(table[j + 1]), tail))
+    nf = 1 << FIXT_BITS
+    fix = [int((d_exp(-Decimal(j) * ln2 / nf) * Decimal(2) ** 63).to_integral_value())
+           for j in range(nf)]
+    out.append("namespace alb {")
+    out.append("constexpr int FIXT_BITS = %d;  // table of 2^FIXT_BITS entries" % FIXT_BITS)
+    out.append("constexpr int FIXT_N = %d;" % nf)
+    out.append("}  // namespace alb")
+    out.append("// 2^63 2^(-j/%d), j = 0..%d, as an initializer list" % (nf, nf - 1))
+    out.append("#define ALB_FIXT_TABLE_VALUES \\")
+    for j in range(0, nf, 4):
+        tail = ", \\" if j < nf - 4 else ""
+        out.append("    " + ", ".join("0x%016xULL" % v for v in fix[j:j + 4]) + tail)
     print("\n".join(out))
 
 
