@@ -101,7 +101,11 @@ typedef struct alb_handle alb_handle; /* opaque */
  *                sender's, multipliers of the previous step moved to the
  *                lattice of the solve; 8 more planes per buffer). The root is
  *                unique, so the start changes only the path and round-off;
- *                ALB_START_MAXWELLIAN follows the oracle's iteration.
+ *                ALB_START_MAXWELLIAN follows the oracle's iteration with
+ *                every step in FP64. The other starts of FP64 plain take the
+ *                iteration's early steps in FP32 (where newton_maxit is at
+ *                least 37) and the last ones, from a residual of about 1e-3
+ *                on, in FP64.
  *   shift_overlap w in [0, 1]: each shift's range widened by w on both
  *                sides, U - n0 - w < u <= U + 1 - n0 + w, so that the ranges
  *                of neighbouring shifts overlap (Sec. III.A.2); 0 (the
@@ -154,13 +158,15 @@ typedef struct {
 typedef struct {
   uint64_t steps;
   uint64_t node_updates;
-  uint64_t newton_iterations;       /* FP64 Newton steps, node and rebuild equilibria */
+  uint64_t newton_iterations;       /* Newton steps of FP64 solves, node and rebuild
+                                       equilibria (FP64 plain: all steps, those in
+                                       fp32_iterations included) */
   uint64_t newton_failures;         /* node equilibria that failed */
   uint64_t reconstructions;         /* missing pulls rebuilt (Grad) */
   uint64_t reconstruction_failures; /* rebuilds that fell back */
   uint64_t newton_calls;            /* equilibrium solves, node and rebuild */
   uint64_t fp64_evaluations;        /* FP64 evaluations of the 21 exponentials */
-  uint64_t fp32_iterations;         /* FP32 Newton steps (FP32 form) */
+  uint64_t fp32_iterations;         /* Newton steps in FP32 */
   uint64_t fp64_updates;            /* FP32 form: residual evaluations that updated
                                        the 21 FP64 populations multiplicatively
                                        after a small step instead of evaluating

@@ -64,6 +64,7 @@ struct Params {
   int warm;          // 1: solves start from the previous step's multipliers
   int rule;          // where ranges overlap: 0 history, 1 neighbourhood
   int moments;       // constraint set: 8, or 4 (reduced model)
+  int mixed64;       // FP64 plain: 1, the early Newton steps run in FP32
   int shakhov;       // 1: Pr != 1, heat-flux term of App. E in the collision
   double nu, gamma, n0, tol;
   double prandtl;    // Pr: tau_Pr = 1/2 + (nu/Pr)/T, kappa = rho Cp nu / Pr

@@ -297,6 +297,12 @@ static cudaError_t launch_step_shape(const FlowDev& f, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// FP64 plain: blocks of 128 threads, two per SM by shared memory, or up to 512^2
+// nodes of 256, where the longer rounds of rebuild solves save more than the
+// second block hides (64^2 vortex 0.39 against 0.42 ms, 201^2 Riemann 0.45 / 0.56,
+// 512^2 shear 1.44 / 1.46, but 700^2 2.53 / 2.46 and 1400^2 vortex 7.73 / 7.39).
+constexpr size_t FP64_SMALL = 512 * 512;
+
 // Block size of the FP32 form: 256 threads, two blocks per SM. Smaller blocks
 // would fill more SMs on a small grid, but an interface tile has then fewer
 // threads for its rebuild solves, which are the longest chain of such a step
@@ -308,7 +314,8 @@ cudaError_t launch_step(FlowDev& f, cudaStream_t s) {
   if (f.q == 49) return launch_step_q49(f, s);
   cudaError_t e;
   if (f.precision == 0)
-    e = launch_step_shape<double, 128, 1>(f, s);
+    e = f.n <= FP64_SMALL && f.prm.ny >= 8 ? launch_step_shape<double, 256, 1>(f, s)
+                                           : launch_step_shape<double, 128, 1>(f, s);
   else if (f.prm.ny >= 8)
     e = launch_step_shape<float, 256, 2>(f, s);
   else

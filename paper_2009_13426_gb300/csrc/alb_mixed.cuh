@@ -142,44 +142,36 @@ __device__ __forceinline__ void load_fixtab(uint64_t* s_fix) {
   for (int j = threadIdx.x; j < FIXT_N; j += blockDim.x) s_fix[j] = g_fixtab[j];
 }
 
-// Exponent e = n >> 8 of the scale 2^(n/N) of the table exponentials below.
-// t = 1.5 * 2^52 + n holds n exactly while |n| < 2^51, and its low word holds n
-// only while |n| < 2^31 (|s| below about 5.8e6); past that the low word wraps,
-// so e is saturated from the high word: 0x43380000 for 0 <= n < 2^32,
-// 0x4337ffff for -2^32 <= n < 0, larger or smaller beyond (also when the
-// rounding trick itself no longer applies). A non-finite t (s NaN or
-// infinite) keeps e in range, so that the NaN of the polynomial comes
-// through. Integer operations only.
-__device__ __forceinline__ int exp_scale_exponent(double t, int n) {
-  const int hi = __double2hiint(t);
-  const bool finite = (hi & 0x7ff00000) != 0x7ff00000;
-  const bool over = hi > 0x43380000 || (hi == 0x43380000 && n < 0);
-  const bool under = hi < 0x4337ffff || (hi == 0x4337ffff && n >= 0);
-  return !finite ? 0 : (over ? 4096 : (under ? -4096 : (n >> EXPT_BITS)));
+// q 2^(n/N) from the table, 0 below 2^-1022 (no subnormal results) and +inf from
+// 2^1024 on; q need not be finite there. Integer operations and one product.
+__device__ __forceinline__ double exp_scaled(double q, int n, const double* tab) {
+  const int e = n >> EXPT_BITS;
+  const int ec = e < -1100 ? -1100 : (e > 1100 ? 1100 : e);  // keeps the shift defined
+  const long long bits = __double_as_longlong(tab[n & (EXPT_N - 1)]) + ((long long)ec << 52);
+  const double v = q * __longlong_as_double(bits);
+  return e < -1022 ? 0.0 : (e > 1023 ? __longlong_as_double(0x7ff0000000000000LL) : v);
 }
 
 // Table-driven FP64 exp(-s) (Tang's method with an N = 256 table): n nearest
-// to -s N / ln2, r = -s - n ln2/N in two parts (|r| <= ln2/512), exp(r) by its
-// degree-4 Taylor polynomial, times 2^(n/N) = 2^(n >> 8) tab[n & 255].
-// 9 FP64 operations. Returns 0 below 2^-1022 (no subnormal results) and +inf
-// from 2^1024 on, for any finite s.
+// to -s N / ln2, r = -s - n ln2/N in two parts, exp(r) by its degree-4 Taylor
+// polynomial, times 2^(n/N) = 2^(n >> 8) tab[n & 255].
+// n comes from an FP32 copy of s: within |s| <= 745 (past which the result is 0
+// or +inf anyway) FP32 holds s N / ln2 to 0.02, so n is the nearest integer or
+// its neighbour near a tie, |r| <= 0.52 ln2/256, and the polynomial's remainder
+// stays below 5e-17. The copy, n and its way back run on the integer pipe: 7 FP64
+// operations (9 with the index rounded in FP64). Past |s| of 5.8e6 the
+// float-to-int rounding saturates and the limits hold; a NaN gives n = 0 and
+// passes through the polynomial.
 __device__ __forceinline__ double exp_neg(double s, const double* tab) {
-  const double shifter = 6755399441055744.0;  // 1.5 * 2^52: rounds to an integer
-  const double t = fma(-s, EXPT_INV_L, shifter);
-  const int n = (int)(unsigned)__double2loint(t);
-  const double nd = t - shifter;
+  const int n = __float2int_rn(mul_rn(-cvt_f32_rn(s), (float)EXPT_INV_L));
+  const double nd = cvt_f64(n);
   double r = fma(nd, -EXPT_L_HI, -s);
   r = fma(nd, -EXPT_L_LO, r);
   double q = fma(r, EXPT_C4, EXPT_C3);
   q = fma(q, r, EXPT_C2);
   q = fma(q, r, 1.0);
   q = fma(q, r, 1.0);
-  const int e = exp_scale_exponent(t, n);
-  const long long bits =
-      __double_as_longlong(tab[n & (EXPT_N - 1)]) + ((long long)e << 52);
-  const double v = q * __longlong_as_double(bits);
-  // out of range: the limits themselves (q need not be finite there)
-  return e < -1022 ? 0.0 : (e > 1023 ? __longlong_as_double(0x7ff0000000000000LL) : v);
+  return exp_scaled(q, n, tab);
 }
 
 // exp(-s) for the FP32 form's refinement: the same table, the reduction in
@@ -203,12 +195,7 @@ __device__ __forceinline__ double exp_neg_refine(double s, float s32, const doub
   const double r = fma(cvt_f64(n), -EXPT_L, -s);
   double q = fma(r, EXPT_C2, 1.0);
   q = fma(q, r, 1.0);
-  const int e = n >> EXPT_BITS;
-  const int ec = e < -1100 ? -1100 : (e > 1100 ? 1100 : e);  // keeps the shift defined
-  const long long bits = __double_as_longlong(tab[n & (EXPT_N - 1)]) + ((long long)ec << 52);
-  const double v = q * __longlong_as_double(bits);
-  // out of range: the limits themselves (q need not be finite there)
-  return e < -1022 ? 0.0 : (e > 1023 ? __longlong_as_double(0x7ff0000000000000LL) : v);
+  return exp_scaled(q, n, tab);
 }
 
 // An exponent held twice: in FP64 and in FP32 (the FP32 copy picks the
@@ -242,6 +229,52 @@ __device__ __forceinline__ float exp_fast(float v) {
   float r;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(mul_rn(v, 1.44269504f)));
   return r;
+}
+
+// G = sum p P and H = sum p P P^T (packed lower triangle) from the sums over the
+// speeds (see PassGH32).
+template <typename R>
+__device__ __forceinline__ void assemble_moments(R p0, const R X[7], const R Y[7], const R E[7],
+                                                 const R O[7], const R Py[7], R G[NM], R H[36]) {
+  const R x3 = X[3] + O[3], y3 = Y[3] + Py[3];  // x^3, y^3
+  G[0] = p0 + X[0] + Y[0] + E[0];
+  G[1] = X[1] + O[1];
+  G[2] = Y[1] + Py[1];
+  G[3] = X[2] + E[2];
+  G[4] = O[2];
+  G[5] = Y[2] + E[2];
+  G[6] = x3 + O[3];  // x^3 + x y^2
+  G[7] = y3 + Py[3];
+#pragma unroll
+  for (int k = 0; k < NM; ++k) H[tri(k, 0)] = G[k];
+  H[tri(1, 1)] = G[3];
+  H[tri(2, 1)] = G[4];
+  H[tri(2, 2)] = G[5];
+  H[tri(3, 1)] = x3;
+  H[tri(3, 2)] = Py[3];
+  H[tri(3, 3)] = X[4] + E[4];
+  H[tri(4, 1)] = Py[3];
+  H[tri(4, 2)] = O[3];
+  H[tri(4, 3)] = O[4];
+  H[tri(4, 4)] = E[4];
+  H[tri(5, 1)] = O[3];
+  H[tri(5, 2)] = y3;
+  H[tri(5, 3)] = E[4];
+  H[tri(5, 4)] = O[4];
+  H[tri(5, 5)] = Y[4] + E[4];
+  H[tri(6, 1)] = fma((R)2, E[4], X[4]);
+  H[tri(6, 2)] = (R)2 * O[4];
+  H[tri(6, 3)] = fma((R)2, O[5], X[5]);
+  H[tri(6, 4)] = (R)2 * Py[5];
+  H[tri(6, 5)] = (R)2 * O[5];
+  H[tri(6, 6)] = fma((R)4, E[6], X[6]);
+  H[tri(7, 1)] = (R)2 * O[4];
+  H[tri(7, 2)] = fma((R)2, E[4], Y[4]);
+  H[tri(7, 3)] = (R)2 * Py[5];
+  H[tri(7, 4)] = (R)2 * O[5];
+  H[tri(7, 5)] = fma((R)2, Py[5], Y[5]);
+  H[tri(7, 6)] = (R)4 * O[6];
+  H[tri(7, 7)] = fma((R)4, E[6], Y[6]);
 }
 
 // FP32 pass: F = sum p, G = sum p P and H = sum p P P^T at the visited
@@ -314,45 +347,7 @@ struct PassGH32 {
     }
   }
   __device__ __forceinline__ void assemble(float G[NM], float H[36]) const {
-    const float x3 = X[3] + O[3], y3 = Y[3] + Py[3];    // x^3, y^3
-    G[0] = F();
-    G[1] = X[1] + O[1];
-    G[2] = Y[1] + Py[1];
-    G[3] = X[2] + E[2];
-    G[4] = O[2];
-    G[5] = Y[2] + E[2];
-    G[6] = x3 + O[3];                                   // x^3 + x y^2
-    G[7] = y3 + Py[3];
-#pragma unroll
-    for (int k = 0; k < NM; ++k) H[tri(k, 0)] = G[k];
-    H[tri(1, 1)] = G[3];
-    H[tri(2, 1)] = G[4];
-    H[tri(2, 2)] = G[5];
-    H[tri(3, 1)] = x3;
-    H[tri(3, 2)] = Py[3];
-    H[tri(3, 3)] = X[4] + E[4];
-    H[tri(4, 1)] = Py[3];
-    H[tri(4, 2)] = O[3];
-    H[tri(4, 3)] = O[4];
-    H[tri(4, 4)] = E[4];
-    H[tri(5, 1)] = O[3];
-    H[tri(5, 2)] = y3;
-    H[tri(5, 3)] = E[4];
-    H[tri(5, 4)] = O[4];
-    H[tri(5, 5)] = Y[4] + E[4];
-    H[tri(6, 1)] = fmaf(2.0f, E[4], X[4]);
-    H[tri(6, 2)] = 2.0f * O[4];
-    H[tri(6, 3)] = fmaf(2.0f, O[5], X[5]);
-    H[tri(6, 4)] = 2.0f * Py[5];
-    H[tri(6, 5)] = 2.0f * O[5];
-    H[tri(6, 6)] = fmaf(4.0f, E[6], X[6]);
-    H[tri(7, 1)] = 2.0f * O[4];
-    H[tri(7, 2)] = fmaf(2.0f, E[4], Y[4]);
-    H[tri(7, 3)] = 2.0f * Py[5];
-    H[tri(7, 4)] = 2.0f * O[5];
-    H[tri(7, 5)] = fmaf(2.0f, Py[5], Y[5]);
-    H[tri(7, 6)] = 4.0f * O[6];
-    H[tri(7, 7)] = fmaf(4.0f, E[6], Y[6]);
+    assemble_moments(p0, X, Y, E, O, Py, G, H);
   }
 };
 
@@ -717,6 +712,15 @@ __device__ __forceinline__ void shift_multipliers(const R l[NM], R dx, R dy, R o
 // small for the same reason: the last step's direction and length but not its
 // start, and the three inputs instead of the eight targets. *gres is the
 // residual maximum (FP32) at the last evaluated point.
+//
+// FACTOR = false is the prelude of the FP64 plain path: it stops, without a
+// factor, at the first point from which the predicted decrease of the dual lies
+// below FP32's resolution (residuals around 1e-3) or whose residual is at most
+// 1e-4. That point is one that the Newton iteration itself passes, to FP32's
+// rounding, with two or three steps still to go. One FP32 step more would be
+// 20 % faster, but its rounding then shows in the last step: the tube parted
+// from the oracle by 1.1e-10 in 1000 steps where it stays below 1e-11 so.
+template <bool FACTOR>
 __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int maxit, bool warm,
                                            float lam[NM], Fact32& fc, int* iters, float* gres) {
   enum { START_WARM, START_MAXWELL, TRIAL, RETURNED };
@@ -796,6 +800,7 @@ __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int ma
       gmax = fmaxf(gmax, fabsf(G[k]));
     }
     *gres = gmax;
+    if (!FACTOR && gmax <= 1e-4f) break;
     if (!isfinite(gmax) || !factor32(H, fc)) return NEWTON_SINGULAR;
     // FP32 exit at 1e-6, five times the FP32 residual's own noise (about
     // 2e-7): below that the FP32 steps only chase rounding, and the
@@ -805,10 +810,11 @@ __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int ma
     gd = 0.0f;
 #pragma unroll
     for (int k = 0; k < NM; ++k) gd = fmaf(G[k], dl[k], gd);
-    if (!(gd > 0.0f)) break;
+    const bool near = gd <= mul_rn(2e-6f, fmaxf(1.0f, fabsf(Fd)));
+    if (!(gd > 0.0f) || (!FACTOR && near)) break;
 #pragma unroll
     for (int k = 0; k < NM; ++k) lam[k] += dl[k];
-    if (gd <= mul_rn(2e-6f, fmaxf(1.0f, fabsf(Fd)))) {
+    if (near) {
       // The predicted decrease gd/2 of the dual lies below its FP32 resolution:
       // a line search would only compare rounding noise. This close to the root
       // the full Newton step is safe; take it and leave the rest to the
@@ -1137,6 +1143,145 @@ static __device__ __noinline__ int newton_fp64g(double ubx, double uby, double T
   }
 }
 
+// FP64 evaluation with the Jacobian: p_i = exp(-(1 + lambda . P(xi_i))) into the
+// column and the 27 moment sums of PassGH32, from which both G (less the
+// targets) and H follow: 96 operations for the sums, against 68 for the
+// constraint sums alone and 150 more for the entries of the Jacobian.
+struct PassGH64 {
+  double p0, X[7], Y[7], E[7], O[7], Py[7];
+  const double* tab;
+  double* col;
+  int stride;
+  __device__ __forceinline__ PassGH64(const double* t, double* c, int s)
+      : p0(0.0), tab(t), col(c), stride(s) {
+#pragma unroll
+    for (int n = 0; n < 7; ++n) X[n] = Y[n] = E[n] = O[n] = Py[n] = 0.0;
+  }
+  __device__ __forceinline__ double ex(int i, double s) const {
+    const double p = exp_neg(s, tab);
+    col[i * stride] = p;
+    return p;
+  }
+  __device__ __forceinline__ void rest(double s) { p0 = ex(0, s); }
+  template <int A, int AX, int IP, int IM>
+  __device__ __forceinline__ void pair(double sp, double sm) {
+    const double pp = ex(IP, sp), pm = ex(IM, sm);
+    const double S = pp + pm, D = pp - pm;
+    double* M = AX == 0 ? X : Y;
+    constexpr int A2 = A * A;
+    M[0] += S;
+    M[1] = madd(M[1], D, A);
+    M[2] = madd(M[2], S, A2);
+    M[3] = madd(M[3], D, A2 * A);
+    M[4] = madd(M[4], S, A2 * A2);
+    M[5] = madd(M[5], D, A2 * A2 * A);
+    M[6] = madd(M[6], S, A2 * A2 * A2);
+  }
+  template <int A, int IPP, int IMP, int IMM, int IPM>
+  __device__ __forceinline__ void quad(double spp, double smp, double smm, double spm) {
+    const double ppp = ex(IPP, spp), pmp = ex(IMP, smp), pmm = ex(IMM, smm), ppm = ex(IPM, spm);
+    const double Ap = ppp + ppm, Bm = pmp + pmm, Cp = ppp - ppm, Dm = pmp - pmm;
+    const double ee = Ap + Bm, oe = Ap - Bm, eo = Cp + Dm, oo = Cp - Dm;
+    constexpr int A2 = A * A;
+    E[0] += ee;
+    E[2] = madd(E[2], ee, A2);
+    E[4] = madd(E[4], ee, A2 * A2);
+    E[6] = madd(E[6], ee, A2 * A2 * A2);
+    O[1] = madd(O[1], oe, A);
+    O[3] = madd(O[3], oe, A2 * A);
+    O[5] = madd(O[5], oe, A2 * A2 * A);
+    Py[1] = madd(Py[1], eo, A);
+    Py[3] = madd(Py[3], eo, A2 * A);
+    Py[5] = madd(Py[5], eo, A2 * A2 * A);
+    O[2] = madd(O[2], oo, A2);
+    O[4] = madd(O[4], oo, A2 * A2);
+    O[6] = madd(O[6], oo, A2 * A2 * A2);
+  }
+  __device__ __forceinline__ void assemble(double G[NM], double H[36]) const {
+    assemble_moments(p0, X, Y, E, O, Py, G, H);
+  }
+};
+
+// Equilibrium of the FP64 plain path: the Newton iteration of newton_fp64g with
+// its early steps in FP32. The FP32 phase follows the iteration to a residual of
+// about 1e-3; the FP64 steps from there have the residual and the Jacobian in
+// FP64, and each step is solved with the FP32 factor and one correction by the
+// FP64 Jacobian (1e-10 of the step). The FP32 rounding of the point they start
+// from, 1e-7, is squared away by the steps as any other error of it, so that the
+// iteration ends where the one in FP64 throughout ends (the same number of steps,
+// 5.1 a solve on the 1024^2 layer, and the same error against 64-bit results).
+// A step costs 430 operations of the FP64 pipe, which bounds this path, where a
+// step of newton_fp64g costs 910: 11.0 -> 4.7 ms a step of the 1024^2 layer,
+// 5570 -> 2160 FP64 instructions per node, 80 % of the pipe busy.
+// Returns NEWTON_OK with the column and the multipliers (lam: in, the warm
+// start if `warm`), or another status: newton_fp64g then solves from the start.
+// *steps counts the FP64 steps.
+static __device__ __noinline__ int solve_mixed64(double ubx, double uby, double T, double tol,
+                                                 bool warm, const double* tab, double* col,
+                                                 int stride, double lam[NM], int* it32, int* steps,
+                                                 int* evals) {
+  float dl[NM];
+  Fact32 fc;
+  float gres = 0.0f;
+  int st;
+  *it32 = *steps = *evals = 0;
+#pragma unroll
+  for (int k = 0; k < NM; ++k) dl[k] = warm ? cvt_f32_rn(lam[k]) : 0.0f;
+  for (bool w = warm;; w = false) {
+    int it = 0;
+    st = newton_fp32<false>(cvt_f32_rn(ubx), cvt_f32_rn(uby), cvt_f32_rn(T), 30, w, dl, fc, &it,
+                            &gres);
+    *it32 += it;
+    if (st == NEWTON_OK || !w) break;
+  }
+  if (st != NEWTON_OK) return st;
+  double m[NM];
+  targets(ubx, uby, T, m);
+#pragma unroll
+  for (int k = 0; k < NM; ++k) lam[k] = cvt_f64(dl[k]);
+  const float tolf = cvt_f32_rn(tol);
+  float last = INFINITY;
+#pragma unroll 1
+  for (int n = 0;; ++n) {
+    PassGH64 pg(tab, col, stride);
+    visit_groups<double>(lam, pg);
+    *evals += 1;
+    double G[NM], H[36];
+    pg.assemble(G, H);
+    float g32[NM], gmax = 0.0f;
+#pragma unroll
+    for (int k = 0; k < NM; ++k) {
+      G[k] -= m[k];
+      g32[k] = cvt_f32_rn(G[k]);
+      gmax = fmaxf(gmax, fabsf(g32[k]));
+    }
+    if (gmax <= tolf) return NEWTON_OK;
+    // (a NaN residual fails the comparison)
+    if (n >= 6 || !(gmax < last)) return NEWTON_MAXIT;
+    last = gmax;
+    float h32[36];
+#pragma unroll
+    for (int k = 0; k < 36; ++k) h32[k] = cvt_f32_rn(H[k]);
+    if (!factor32(h32, fc)) return NEWTON_SINGULAR;
+    solve32(fc, g32, dl);
+    double d[NM];
+#pragma unroll
+    for (int k = 0; k < NM; ++k) d[k] = cvt_f64(dl[k]);
+    float r32[NM];
+#pragma unroll
+    for (int a = 0; a < NM; ++a) {
+      double r = G[a];
+#pragma unroll
+      for (int b = 0; b < NM; ++b) r = fma(-H[a >= b ? tri(a, b) : tri(b, a)], d[b], r);
+      r32[a] = cvt_f32_rn(r);
+    }
+    solve32(fc, r32, dl);
+#pragma unroll
+    for (int k = 0; k < NM; ++k) lam[k] += d[k] + cvt_f64(dl[k]);
+    *steps += 1;
+  }
+}
+
 // Reduced model (App. C.2, Eq. feqNum_4Mom): four constraints - mass,
 // momentum and the energy trace sum f xi_a xi_a = rho (|ubar|^2 + D T) - and
 // the exponential family in (1, xi_x, xi_y, |xi|^2). The multipliers are kept
@@ -1368,7 +1513,7 @@ __device__ __forceinline__ int solve_fix(double ubx, double uby, double T, float
   int st;
   for (bool w = warm;; w = false) {
     int it32 = 0;
-    st = newton_fp32(ubx32, uby32, T32, 30, w, lam, fc, &it32, &gres);
+    st = newton_fp32<true>(ubx32, uby32, T32, 30, w, lam, fc, &it32, &gres);
     cnt->fp32_iters += it32;
     if (st == NEWTON_OK || !w) break;
   }
@@ -1405,7 +1550,7 @@ static __device__ __noinline__ int equilibrium_mixed(double ubx, double uby, dou
     for (int k = 0; k < NM; ++k) l32[k] = warm[k];
   for (;;) {
     int it32 = 0;
-    st = newton_fp32(ubx32, uby32, T32, 30, w, l32, fc, &it32, &gres);
+    st = newton_fp32<true>(ubx32, uby32, T32, 30, w, l32, fc, &it32, &gres);
     cnt->fp32_iters += it32;
     if (st == NEWTON_OK || !w) break;
     w = false;

@@ -49,8 +49,8 @@ struct Columns {
   }
 };
 
-// Equilibrium of one node in the storage precision P: the full FP64 Newton for
-// the FP64 plain path, FP32 Newton with the fixed-point refinement for the FP32
+// Equilibrium of one node in the storage precision P: FP32 Newton steps and FP64
+// residuals for the FP64 plain path (or all FP64 steps: Params::mixed64), FP32 Newton with the fixed-point refinement for the FP32
 // form (FP64 refinement where that does not reach), both started from the
 // multipliers in lam (precision P) if `warm` is set. The equilibrium per unit
 // density lands in the thread's column (Q63 instead of FP64 where *fixed is
@@ -102,10 +102,22 @@ __device__ __forceinline__ int node_equilibrium(const Params& pr, const Columns<
   } else {
     int it = 0, ev = 0;
     double l64[NM];
-    st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l64, &it, &ev,
-                      warm ? w : nullptr);
-    cnt->fp64_iters += it;
-    cnt->fp64_evals += ev;
+    st = NEWTON_SINGULAR;
+    if (pr.mixed64) {
+      int it32 = 0;
+#pragma unroll
+      for (int k = 0; k < NM; ++k) l64[k] = lam[k];
+      st = solve_mixed64(ubx, uby, T, pr.tol, warm, cl.exptab, cl.eq, B, l64, &it32, &it, &ev);
+      cnt->fp32_iters += it32;
+      cnt->fp64_iters += it32 + it;
+      cnt->fp64_evals += ev;
+    }
+    if (st != NEWTON_OK) {
+      st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l64, &it, &ev,
+                        warm ? w : nullptr);
+      cnt->fp64_iters += it;
+      cnt->fp64_evals += ev;
+    }
     if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
       // the previous multipliers led nowhere: start again from the Maxwellian
       st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l64, &it, &ev, nullptr);
