@@ -113,7 +113,8 @@ typedef struct alb_handle alb_handle; /* opaque */
  *   moments      constraint set of the numerical equilibrium: 8 (Eqs.
  *                G0_8mom..G3yaa_8mom, the default) or 4 (the reduced model
  *                of App. C.2, Eq. feqNum_4Mom: mass, momentum and the energy
- *                trace; a 4x4 FP64 Newton in both precisions) on D2Q21; 13
+ *                trace; solved as the full set is in the FP32 form, by a 4x4
+ *                Newton in FP64 in FP64 plain) on D2Q21; 13
  *                (Eqs. G0..G4yyaa: moments up to third order and the trace
  *                of the fourth, Eq. feqNum_13Mom with the x^3 monomial the
  *                printed exponent omits) on D2Q49.

@@ -67,23 +67,42 @@ __device__ __forceinline__ int node_equilibrium(const Params& pr, const Columns<
   for (int k = 0; k < NM; ++k) w[k] = lam[k];
   int st;
   if (pr.moments == 4) {
-    // reduced model: FP64 4x4 Newton in both precisions
-    double w8[NM], l8[NM];
-    if (warm)
-#pragma unroll
-      for (int k = 0; k < NM; ++k) w8[k] = (double)lam[k];
+    // reduced model: in the FP32 form as the full one, else (and where that
+    // does not reach) an FP64 4x4 Newton
     int it = 0, ev = 0;
-    st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l8, &it, &ev,
-                       warm ? w8 : nullptr);
-    cnt->fp64_iters += it;
-    cnt->fp64_evals += ev;
-    if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
-      st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l8, &it, &ev, nullptr);
+    st = NEWTON_SINGULAR;
+    if constexpr (std::is_same<P, float>::value) {
+      int it32 = 0, up = 0;
+      float l32[NM];
+#pragma unroll
+      for (int k = 0; k < NM; ++k) l32[k] = lam[k];
+      st = solve4_fix(ubx, uby, T, (float)pr.tol, warm, cl.fixtab,
+                      reinterpret_cast<uint64_t*>(cl.eq), B, l32, &it32, &ev, &up);
+      cnt->fp32_iters += it32;
+      cnt->fp64_evals += ev;
+      cnt->fp64_updates += up;
+      *fixed = st == NEWTON_OK;
+      if (st == NEWTON_OK)
+#pragma unroll
+        for (int k = 0; k < NM; ++k) lam[k] = l32[k];
+    }
+    if (st != NEWTON_OK) {
+      double w8[NM], l8[NM];
+#pragma unroll
+      for (int k = 0; k < NM; ++k) w8[k] = warm ? (double)lam[k] : 0.0;
+      st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l8, &it, &ev,
+                         warm ? w8 : nullptr);
       cnt->fp64_iters += it;
       cnt->fp64_evals += ev;
-    }
+      if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
+        st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l8, &it, &ev,
+                           nullptr);
+        cnt->fp64_iters += it;
+        cnt->fp64_evals += ev;
+      }
 #pragma unroll
-    for (int k = 0; k < NM; ++k) lam[k] = (P)l8[k];
+      for (int k = 0; k < NM; ++k) lam[k] = (P)l8[k];
+    }
   } else if constexpr (std::is_same<P, float>::value) {
     st = solve_fix(ubx, uby, T, (float)pr.tol, warm, cl.fixtab, reinterpret_cast<uint64_t*>(cl.eq),
                    B, lam, cnt);
