@@ -5,7 +5,7 @@
 // 13-moment equilibrium of Eqs. G0..G4yyaa / feqNum_13Mom. FP64 throughout.
 //
 // Velocity i = (x, y) has index i = (x + 3) + 7 (y + 3). One thread per node;
-// a block is a row segment of B nodes. Each thread owns two columns of the
+// a block is a tile of 8 x 8 nodes. Each thread owns two columns of the
 // block's dynamic shared memory (stride B): its 98 pulled populations and the
 // 49 equilibrium values per unit density of its latest solve. A missing pull
 // needs the equilibrium of its sender's state in the receiver's lattice; the
@@ -13,7 +13,8 @@
 // threads, and forms the pulls from the multipliers (see step_kernel).
 // Exponentials use the table-driven FP64 exp of the D2Q21 kernels.
 //
-// Newton on the 13 multipliers follows the 8-moment solver's iteration
+// Newton on the 13 multipliers (early steps in FP32, solve13_mixed; newton13 is
+// the iteration with every step in FP64) follows the 8-moment solver's iteration
 // (Maxwellian start with lambda_0 from the normalisation, exact Jacobian,
 // Armijo backtracking on the convex dual, stop at max|G|/rho <= tol). The
 // Jacobian entries are moments sum_i p_i x^a y^b with a + b <= 8; the lattice
@@ -259,6 +260,298 @@ __device__ __noinline__ int newton13(double ubx, double uby, double T, double to
   return status;
 }
 
+// ------------------------------------------------- mixed-precision solve
+//
+// The iteration of newton13 with its early steps in FP32 (see solve_mixed64 of
+// the D2Q21 solver): FP32 down to a residual of about 1e-3, then residual,
+// moments and multipliers in FP64, each step solved with the FP32 factor and one
+// correction by the FP64 Jacobian.
+//
+// One pass evaluates the 49 exponents, the exponentials and the 45 moments M_ab =
+// sum p x^a y^b, a + b <= 8, through the parities of the tensor-product lattice:
+// the exponent of a row is a polynomial in x whose even and odd parts serve +-x,
+// its coefficients' even and odd parts in y serve +-y, and the sums run over the
+// same pairs. 610 operations for exponents and sums, where velocity by velocity
+// they are 540 and 664; FP64 operations a Newton step, all in all, 3740 -> 1300.
+// With the 8 x 8 tiles below: 35.6 -> 1.86 ms a step of the 192^2 shear layer.
+__device__ __forceinline__ float exp_of(float s, const double*) { return exp_fast(-s); }
+__device__ __forceinline__ double exp_of(double s, const double* tab) { return exp_neg(s, tab); }
+__device__ __forceinline__ void put(double* eq, int i, double p) { eq[i * B] = p; }
+__device__ __forceinline__ void put(double*, int, float) {}
+
+// Index of M_ab in the packed list (a + b <= 8).
+__host__ __device__ constexpr int mi(int a, int b) { return 9 * a - a * (a - 1) / 2 + b; }
+constexpr int NMOM = 45;
+
+template <typename R>
+__device__ __forceinline__ R fma_i(R v, int c, R s) {
+  return c == 1 ? s + v : fma(v, (R)c, s);
+}
+
+// One row's populations from its coefficients c0..c4, and its sums S_a = sum p x^a.
+template <typename R>
+__device__ __forceinline__ void row_pass(const R c[5], int y, const double* tab, double* eq,
+                                         R S[9]) {
+  const R p0 = exp_of(c[0], tab);
+  put(eq, 3 + 7 * (y + 3), p0);
+  S[0] = p0;
+#pragma unroll
+  for (int a = 1; a < 9; ++a) S[a] = (R)0;
+#pragma unroll
+  for (int x = 1; x <= 3; ++x) {
+    const R e = fma_i(c[4], x * x * x * x, fma_i(c[2], x * x, c[0]));
+    const R o = fma_i(c[3], x * x * x, x == 1 ? c[1] : mul_rn(c[1], (R)x));
+    const R pp = exp_of(e + o, tab), pm = exp_of(e - o, tab);
+    put(eq, 3 + x + 7 * (y + 3), pp);
+    put(eq, 3 - x + 7 * (y + 3), pm);
+    const R E = pp + pm, D = pp - pm;
+#pragma unroll
+    for (int a = 0; a < 9; ++a) S[a] = fma_i(a % 2 ? D : E, ipow(x, a), S[a]);
+  }
+}
+
+template <typename R>
+__device__ __forceinline__ void pass13(const R l[M], const double* tab, double* eq, R mom[NMOM]) {
+#pragma unroll
+  for (int k = 0; k < NMOM; ++k) mom[k] = (R)0;
+  {
+    const R c[5] = {(R)1 + l[0], l[1], l[3], l[6], l[10]};
+    R S[9];
+    row_pass(c, 0, tab, eq, S);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) mom[mi(a, 0)] = S[a];
+  }
+#pragma unroll
+  for (int y = 1; y <= 3; ++y) {
+    const R e0 = fma_i(l[12], y * y * y * y, fma_i(l[5], y * y, (R)1 + l[0]));
+    const R o0 = fma_i(l[9], y * y * y, y == 1 ? l[2] : mul_rn(l[2], (R)y));
+    const R e1 = fma_i(l[8], y * y, l[1]);
+    const R o1 = fma_i(l[11], y * y * y, y == 1 ? l[4] : mul_rn(l[4], (R)y));
+    const R e2 = fma_i(l[10] + l[12], y * y, l[3]);
+    const R o2 = y == 1 ? l[7] : mul_rn(l[7], (R)y);
+    const R o3 = y == 1 ? l[11] : mul_rn(l[11], (R)y);
+    const R cp[5] = {e0 + o0, e1 + o1, e2 + o2, l[6] + o3, l[10]};
+    const R cm[5] = {e0 - o0, e1 - o1, e2 - o2, l[6] - o3, l[10]};
+    R Sp[9], Sm[9];
+    row_pass(cp, y, tab, eq, Sp);
+    row_pass(cm, -y, tab, eq, Sm);
+#pragma unroll
+    for (int a = 0; a < 9; ++a) {
+      const R E = Sp[a] + Sm[a], D = Sp[a] - Sm[a];
+#pragma unroll
+      for (int b = 0; a + b < 9; ++b)
+        mom[mi(a, b)] = fma_i(b % 2 ? D : E, ipow(y, b), mom[mi(a, b)]);
+    }
+  }
+}
+
+// sum p P_k, and the Jacobian's entry sum p P_r P_c, from the moments.
+template <typename R>
+__device__ __forceinline__ R sum_of(const R mom[NMOM], int k) {
+  R s = mom[mi(term(k, 0).a, term(k, 0).b)];
+  if (nterms(k) == 2) s += mom[mi(term(k, 1).a, term(k, 1).b)];
+  return s;
+}
+template <typename R>
+__device__ __forceinline__ R jac_of(const R mom[NMOM], int r, int c) {
+  R s = (R)0;
+#pragma unroll
+  for (int t = 0; t < nterms(r); ++t)
+#pragma unroll
+    for (int u = 0; u < nterms(c); ++u) {
+      const R v = mom[mi(term(r, t).a + term(c, u).a, term(r, t).b + term(c, u).b)];
+      s = t + u == 0 ? v : s + v;
+    }
+  return s;
+}
+
+// FP32 Cholesky factor (reciprocal diagonal) of the Jacobian, in place, and the
+// solves with it.
+__device__ __forceinline__ bool factor13(float H[M * (M + 1) / 2]) {
+  bool ok = true;
+#pragma unroll
+  for (int j = 0; j < M; ++j) {
+    float d = H[tri(j, j)];
+#pragma unroll
+    for (int k = 0; k < j; ++k) d = fmaf(-H[tri(j, k)], H[tri(j, k)], d);
+    ok = ok && d > 0.0f;
+    const float il = rsqrt_fast(fmaxf(d, 1e-30f));
+    H[tri(j, j)] = il;
+#pragma unroll
+    for (int i = j + 1; i < M; ++i) {
+      float t = H[tri(i, j)];
+#pragma unroll
+      for (int k = 0; k < j; ++k) t = fmaf(-H[tri(i, k)], H[tri(j, k)], t);
+      H[tri(i, j)] = mul_rn(t, il);
+    }
+  }
+  return ok;
+}
+__device__ __forceinline__ void solve13(const float L[M * (M + 1) / 2], const float g[M],
+                                        float d[M]) {
+#pragma unroll
+  for (int i = 0; i < M; ++i) {
+    float t = g[i];
+#pragma unroll
+    for (int k = 0; k < i; ++k) t = fmaf(-L[tri(i, k)], d[k], t);
+    d[i] = mul_rn(t, L[tri(i, i)]);
+  }
+#pragma unroll
+  for (int i = M - 1; i >= 0; --i) {
+    float t = d[i];
+#pragma unroll
+    for (int k = i + 1; k < M; ++k) t = fmaf(-L[tri(k, i)], d[k], t);
+    d[i] = mul_rn(t, L[tri(i, i)]);
+  }
+}
+
+// FP32 phase from the Maxwellian; false if it fails.
+__device__ __noinline__ bool prelude13(float ubx, float uby, float T, float l[M], int* iters) {
+  float m[M];
+  {
+    double md[M];
+    targets13(ubx, uby, T, md);
+#pragma unroll
+    for (int k = 0; k < M; ++k) m[k] = cvt_f32_rn(md[k]);
+  }
+  const float iT = 1.0f / T;
+#pragma unroll
+  for (int k = 0; k < M; ++k) l[k] = 0.0f;
+  l[1] = -ubx * iT;
+  l[2] = -uby * iT;
+  l[3] = 0.5f * iT;
+  l[5] = 0.5f * iT;
+  float d[M], Fd = 0.0f, gd = 0.0f, t = 1.0f;
+  int ls = 0, it = 0;
+  bool start = true;
+#pragma unroll 1
+  for (;;) {
+    float mom[NMOM];
+    pass13<float>(l, nullptr, nullptr, mom);
+    if (start) {
+      const float z = mom[0], iz = 1.0f / z;
+      l[0] = logf(z);
+#pragma unroll
+      for (int k = 0; k < NMOM; ++k) mom[k] *= iz;
+    }
+    float F = mom[0];
+#pragma unroll
+    for (int k = 0; k < M; ++k) F = fmaf(l[k], m[k], F);
+    if (!start) {
+      if (!(isfinite(F) && F <= fmaf(4e-7f, fabsf(Fd), fmaf(-1e-4f * t, gd, Fd)))) {
+        if (++ls >= 12) return false;
+        t *= 0.5f;
+#pragma unroll
+        for (int k = 0; k < M; ++k) l[k] = fmaf(-t, d[k], l[k]);
+        continue;
+      }
+      ++it;
+    }
+    start = false;
+    Fd = F;
+    float g[M], H[M * (M + 1) / 2], gmax = 0.0f;
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+      g[k] = sum_of(mom, k) - m[k];
+      gmax = fmaxf(gmax, fabsf(g[k]));
+    }
+    *iters = it;
+    if (!isfinite(gmax)) return false;
+    if (gmax <= 1e-4f) return true;
+    if (it >= 30) return false;
+#pragma unroll
+    for (int r = 0; r < M; ++r)
+#pragma unroll
+      for (int c = 0; c <= r; ++c) H[tri(r, c)] = jac_of(mom, r, c);
+    if (!factor13(H)) return false;
+    solve13(H, g, d);
+    gd = 0.0f;
+#pragma unroll
+    for (int k = 0; k < M; ++k) gd = fmaf(g[k], d[k], gd);
+    if (!(gd > 0.0f)) return false;
+    if (gd <= 2e-6f * fmaxf(1.0f, fabsf(Fd))) return true;
+#pragma unroll
+    for (int k = 0; k < M; ++k) l[k] += d[k];
+    t = 1.0f;
+    ls = 0;
+  }
+}
+
+// As newton13; *iters counts all steps. A status other than NEWTON_OK leaves the
+// solve to newton13.
+__device__ __noinline__ int solve13_mixed(double ubx, double uby, double T, double tol, double* eq,
+                                          const double* tab, double lam[M], int* iters) {
+  *iters = 0;
+  if (!(T > 0.0) || !isfinite(T) || !isfinite(ubx) || !isfinite(uby)) return NEWTON_UNREALIZABLE;
+  {
+    float l32[M];
+    if (!prelude13(cvt_f32_rn(ubx), cvt_f32_rn(uby), cvt_f32_rn(T), l32, iters)) return SINGULAR;
+#pragma unroll
+    for (int k = 0; k < M; ++k) lam[k] = cvt_f64(l32[k]);
+  }
+  const float tolf = cvt_f32_rn(tol);
+  float last = INFINITY;
+#pragma unroll 1
+  for (int n = 0;; ++n) {
+    double mom[NMOM], G[M], m[M];
+    pass13<double>(lam, tab, eq, mom);
+    targets13(ubx, uby, T, m);
+    float g32[M], gmax = 0.0f;
+#pragma unroll
+    for (int k = 0; k < M; ++k) {
+      G[k] = sum_of(mom, k) - m[k];
+      g32[k] = cvt_f32_rn(G[k]);
+      gmax = fmaxf(gmax, fabsf(g32[k]));
+    }
+    if (gmax <= tolf) return OK;
+    if (n >= 6 || !(gmax < last)) return MAXIT;
+    last = gmax;
+    float L[M * (M + 1) / 2], d32[M], r32[M];
+    {
+      float m32[NMOM];
+#pragma unroll
+      for (int k = 0; k < NMOM; ++k) m32[k] = cvt_f32_rn(mom[k]);
+#pragma unroll
+      for (int r = 0; r < M; ++r)
+#pragma unroll
+        for (int c = 0; c <= r; ++c) L[tri(r, c)] = jac_of(m32, r, c);
+    }
+    if (!factor13(L)) return SINGULAR;
+    solve13(L, g32, d32);
+    double d[M];
+#pragma unroll
+    for (int k = 0; k < M; ++k) d[k] = cvt_f64(d32[k]);
+#pragma unroll
+    for (int r = 0; r < M; ++r)
+#pragma unroll
+      for (int c = 0; c <= r; ++c) {
+        const double h = jac_of(mom, r, c);
+        G[r] = fma(-h, d[c], G[r]);
+        if (c < r) G[c] = fma(-h, d[r], G[c]);
+      }
+#pragma unroll
+    for (int k = 0; k < M; ++k) r32[k] = cvt_f32_rn(G[k]);
+    solve13(L, r32, d32);
+#pragma unroll
+    for (int k = 0; k < M; ++k) lam[k] += d[k] + cvt_f64(d32[k]);
+    *iters += 1;
+  }
+}
+
+// The solve of the step and of the initial state: mixed precision, newton13
+// where that fails or is not asked for (Params::mixed64).
+__device__ __forceinline__ int solve13(const Params& pr, double ubx, double uby, double T,
+                                       double* eq, const double* tab, double lam[M], int* iters) {
+  int st = SINGULAR;
+  if (pr.mixed64) st = solve13_mixed(ubx, uby, T, pr.tol, eq, tab, lam, iters);
+  if (st != OK && st != NEWTON_UNREALIZABLE) {
+    int it = 0;
+    st = newton13(ubx, uby, T, pr.tol, pr.maxit, eq, tab, lam, &it);
+    *iters = it;
+  }
+  return st;
+}
+
 struct Count {
   unsigned iters = 0, calls = 0, fail = 0, rec = 0, rec_fail = 0;
 };
@@ -343,8 +636,7 @@ __device__ __noinline__ int sender_solve(const Params pr, const Sender s, int Up
                                          double* eq, const double* tab, double lam[M],
                                          Count* cnt) {
   int it = 0;
-  const int st = s.rho > 0.0 ? newton13(s.ux - Upx, s.uy - Upy, s.T, pr.tol, pr.maxit, eq, tab,
-                                        lam, &it)
+  const int st = s.rho > 0.0 ? solve13(pr, s.ux - Upx, s.uy - Upy, s.T, eq, tab, lam, &it)
                              : NEWTON_UNREALIZABLE;
   cnt->iters += it;
   cnt->calls += 1;
@@ -407,8 +699,7 @@ __device__ __forceinline__ void collide(const Params& pr, const double* col, dou
                           : lat_code(select_shift_kept(ux, Ux, pr), select_shift_kept(uy, Uy, pr));
   double lam[M];
   int it = 0;
-  const int ns = rho > 0.0 ? newton13(ubx, uby, T, pr.tol, pr.maxit, eq, tab, lam, &it)
-                           : NEWTON_UNREALIZABLE;
+  const int ns = rho > 0.0 ? solve13(pr, ubx, uby, T, eq, tab, lam, &it) : NEWTON_UNREALIZABLE;
   cnt->iters += it;
   cnt->calls += 1;
   if (ns == NEWTON_OK) {
@@ -481,12 +772,15 @@ __device__ __forceinline__ void flush(unsigned long long* ctr, const Count& c) {
 // so neither the order of insertion nor the solving thread changes it.
 constexpr int HCAP = 512;        // hash positions per block (power of two)
 constexpr int SCAP = 192;        // distinct solves kept per block
-constexpr int KW = B + 12;       // sender x offsets: x0 - 6 .. x0 + B + 5
+// A square tile's missing pulls share more senders than a row's (1.48 against
+// 1.78 solves per node on the 192^2 layer), and its solves fill fewer rounds.
+constexpr int TW = 8, TH = B / TW;  // tile of a block's nodes
+constexpr int KW = TW + 12;      // sender x offsets: x0 - 6 .. x0 + TW + 5
 constexpr unsigned EMPTY = 0xffffffffu;
 constexpr unsigned short NOSLOT = 0xffff;
 
-__device__ __forceinline__ unsigned rebuild_key(int sx, int sy, int x0, int y, int code) {
-  return (unsigned)(((sy - y + 6) * KW + (sx - x0 + 6)) * 49 + code);
+__device__ __forceinline__ unsigned rebuild_key(int sx, int sy, int x0, int y0, int code) {
+  return (unsigned)(((sy - y0 + 6) * KW + (sx - x0 + 6)) * 49 + code);
 }
 
 __global__ void __launch_bounds__(B) step_kernel(StepArgs<double> a) {
@@ -507,9 +801,9 @@ __global__ void __launch_bounds__(B) step_kernel(StepArgs<double> a) {
   double* eq = smem49 + NP * B + t;
   const Params& pr = a.prm;
   const size_t ps = a.ps;
-  const int x0 = blockIdx.x * B, y = blockIdx.y;
-  const int x = x0 + t;
-  const bool active = x < pr.nx;
+  const int x0 = blockIdx.x * TW, y0 = blockIdx.y * TH;
+  const int x = x0 + t % TW, y = y0 + t / TW;
+  const bool active = x < pr.nx && y < pr.ny;
   Count cnt;
   size_t k = 0;
   int code = 0;
@@ -529,7 +823,7 @@ __global__ void __launch_bounds__(B) step_kernel(StepArgs<double> a) {
         continue;
       }
       missing |= 1ull << i;
-      const unsigned key = rebuild_key(sx, sy, x0, y, code);
+      const unsigned key = rebuild_key(sx, sy, x0, y0, code);
       unsigned short pos = NOSLOT;
       unsigned h = (key * 2654435761u) >> 23;  // 9 bits: HCAP = 512
       for (int probe = 0; probe < HCAP; ++probe, h = (h + 1) & (HCAP - 1)) {
@@ -555,7 +849,7 @@ __global__ void __launch_bounds__(B) step_kernel(StepArgs<double> a) {
   for (int e = t; e < ns; e += B) {
     const unsigned key = s_skey[e];
     const int c = (int)(key % 49u), off = (int)(key / 49u);
-    const int sx = x0 + off % KW - 6, sy = y + off / KW - 6;
+    const int sx = x0 + off % KW - 6, sy = y0 + off / KW - 6;
     const Sender snd = sender_state(pr, a.mom_in, ps, sx, sy);
     double lam[M];
     const int st = sender_solve(pr, snd, lat_ux(c), lat_uy(c), eq, s_tab, lam, &cnt);
@@ -652,7 +946,7 @@ __global__ void __launch_bounds__(B) init_kernel(InitArgs49 a) {
     const bool ok = (r > 0.0) && (T > 0.0) && isfinite(r) && isfinite(T);
     double lam[M];
     int it = 0;
-    const int ns = ok ? newton13(ux - U0x, uy - U0y, T, pr.tol, pr.maxit, eq, s_tab, lam, &it)
+    const int ns = ok ? solve13(pr, ux - U0x, uy - U0y, T, eq, s_tab, lam, &it)
                       : NEWTON_UNREALIZABLE;
     if (!ok) bad += 1;
     if (ok && ns != NEWTON_OK) cnt.fail += 1;
@@ -721,6 +1015,9 @@ __global__ void __launch_bounds__(B)
 }
 
 static dim3 grid_of(const Params& p) { return dim3((p.nx + B - 1) / B, p.ny); }
+static dim3 tiles_of(const Params& p) {
+  return dim3((p.nx + TW - 1) / TW, (p.ny + TH - 1) / TH);
+}
 
 }  // namespace q49
 
@@ -744,7 +1041,7 @@ cudaError_t launch_step_q49(FlowDev& f, cudaStream_t s) {
                                        cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)q49::SMEM);
   if (e != cudaSuccess) return e;
-  q49::step_kernel<<<q49::grid_of(f.prm), q49::B, q49::SMEM, s>>>(a);
+  q49::step_kernel<<<q49::tiles_of(f.prm), q49::B, q49::SMEM, s>>>(a);
   e = cudaGetLastError();
   if (e == cudaSuccess) f.cur = out;
   return e;
