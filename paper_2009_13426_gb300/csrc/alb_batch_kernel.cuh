@@ -22,12 +22,11 @@ __global__ void __launch_bounds__(B, MINB)
   static_assert(sizeof(StepArgs<P>) % 8 == 0, "step arguments copy as 8-byte words");
   static_assert(sizeof(StepArgs<P>) / 8 <= B, "one word per thread");
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double s_tab[EXPT_N];
   __shared__ __align__(16) unsigned long long s_args[sizeof(StepArgs<P>) / 8];
   __shared__ int s_item;
-  __shared__ RebuildQueue<B> s_rq;
+  __shared__ RebuildQueue<P, B> s_rq;
   const StepArgs<P>& a = *reinterpret_cast<const StepArgs<P>*>(s_args);
-  const Columns<P, B> cl(smem_raw, s_tab);  // includes a barrier
+  const Columns<P, B> cl(smem_raw);  // includes a barrier
   int it = blockIdx.x;
   int loaded = -1;  // (flow, buffer) whose arguments s_args holds
   for (;;) {
@@ -52,7 +51,7 @@ __global__ void __launch_bounds__(B, MINB)
       __syncthreads();
       loaded = want;
     }
-    NodeCount nc;
+    NodeCount<P> nc;
     tile_step<P, B>(a, w.x0, w.y0, w.tw_log2, cl, s_rq, nc);
     flush_counts(a.ctr, nc);
     if (!counter) it += gridDim.x;

@@ -37,7 +37,7 @@ constexpr uint32_t FIX_Y_END = (uint32_t)FIX_OCTAVES << FIX_BITS;
 constexpr float FIX_SCALE = 48408812.0f;  // 2^25 / ln 2
 // Exponents above this magnitude (44 < 64 ln 2) could wrap in 32 bits.
 constexpr float FIX_S_MAX = 44.0f;
-// Largest step whose factor exp(-d) - 1 fits the 23-bit rounding below.
+// Largest step taken multiplicatively (the factor's polynomial: 3e-14).
 constexpr float FIX_STEP_MAX = 9e-4f;
 static_assert(FIXT_BITS == 9, "the index and remainder below assume 512 table entries");
 
@@ -70,15 +70,15 @@ ALB_CVT_FN uint64_t fix_exp(uint32_t y, const uint64_t* tab) {
 
 // Scale of the factors of one multiplicative update whose exponent changes are
 // all at most `bound` (<= FIX_STEP_MAX) in magnitude: e = exp(-d) - 1 in units of
-// 2^-(32 + k), k as large as 22 bits of magnitude allow, so that the rounding
-// of e is 2^-22 of the bound and a sequence of shrinking steps converges.
+// 2^-(32 + k), k as large as 31 bits of magnitude allow, so that e keeps its FP32
+// precision and a sequence of shrinking steps converges.
 struct FixStep {
   float c1, c2, c3;  // e 2^(32 + k) = c1 d + c2 d^2 + c3 d^3
   uint32_t k;
 };
 ALB_CVT_FN FixStep fix_step(float bound) {
   const int eb = (int)(cvt_bits_f32(bound) >> 23) - 127;  // bound < 2^(eb + 1)
-  int k = -12 - eb;
+  int k = -3 - eb;
   k = k < 0 ? 0 : (k > 31 ? 31 : k);
   const float s = cvt_f32_of_bits((uint32_t)(127 + 32 + k) << 23);  // 2^(32 + k)
   return FixStep{-s, 0.5f * s, -0.16666667f * s, (uint32_t)k};
@@ -86,10 +86,13 @@ ALB_CVT_FN FixStep fix_step(float bound) {
 
 // Q63 population P times exp(-d) (the factor by a degree-3 polynomial in FP32).
 ALB_CVT_FN uint64_t fix_scale(uint64_t P, float d, const FixStep& c) {
-  // e 2^(32 + k), below 2^22 in magnitude; added to 1.5 * 2^23 it is rounded to
-  // an integer in the low bits
-  const float q = fmaf(d, fmaf(d, fmaf(d, c.c3, c.c2), c.c1), 12582912.0f);
-  const int e = (int)(cvt_bits_f32(q) - 0x4b400000u);
+  // e 2^(32 + k), below 2^31 in magnitude, rounded to an integer
+  const float q = d * fmaf(d, fmaf(d, c.c3, c.c2), c.c1);
+#ifdef __CUDA_ARCH__
+  const int e = __float2int_rn(q);
+#else
+  const int e = (int)lrintf(q);
+#endif
   const uint32_t lo = (uint32_t)P, hi = (uint32_t)(P >> 32);
 #ifdef __CUDA_ARCH__
   const uint32_t w = __umulhi(lo, (uint32_t)e);

@@ -25,10 +25,9 @@ template <typename P, int B, int MINB>
 __global__ void __launch_bounds__(B, MINB)
     step_kernel(const __grid_constant__ StepArgs<P> a, int lg) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double s_tab[EXPT_N];
-  __shared__ RebuildQueue<B> s_rq;
-  const Columns<P, B> cl(smem_raw, s_tab);  // includes a barrier
-  NodeCount nc;
+  __shared__ RebuildQueue<P, B> s_rq;
+  const Columns<P, B> cl(smem_raw);  // includes a barrier
+  NodeCount<P> nc;
   tile_step<P, B>(a, blockIdx.x << lg, blockIdx.y * (B >> lg), lg, cl, s_rq, nc);
   flush_counts(a.ctr, nc);
 }
@@ -62,13 +61,12 @@ template <typename P>
 __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1))
     init_kernel(const __grid_constant__ InitArgs<P> a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double s_tab[EXPT_N];
-  const Columns<P, BLOCK> cl(smem_raw, s_tab);
+  const Columns<P, BLOCK> cl(smem_raw);
   const Params& pr = a.prm;
   const int x = blockIdx.x * BLOCK + threadIdx.x;
   const int y = blockIdx.y;
   unsigned n_bad = 0, n_fail = 0;
-  SolveCount cnt;
+  NodeCount<P> cnt;  // (the initial solves are not step work: only failures are counted)
   if (x < pr.nx) {
     const size_t nx = (size_t)pr.nx;
     const size_t k = (size_t)y * nx + x;
@@ -93,9 +91,11 @@ __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1)
     P lam[NM];
     const bool realizable = (r > 0.0) && (T > 0.0) && isfinite(r) && isfinite(T);
     bool fixed = false;
-    const int ns = realizable ? node_equilibrium<P, BLOCK>(pr, cl, ux - U0x, uy - U0y, T, false,
-                                                           lam, &cnt, &fixed)
-                              : NEWTON_UNREALIZABLE;
+    const NodeState s0{r, ux - U0x, uy - U0y, T, 0};
+    const int ns = realizable
+                       ? node_equilibrium<P, BLOCK>(pr, cl, s0, false, [](P*) {}, lam, &cnt, nullptr,
+                                                    &fixed)
+                       : NEWTON_UNREALIZABLE;
     if (!realizable) n_bad += 1;
     if (ns != NEWTON_OK && realizable) n_fail += 1;
     const double gfac = (2.0 * pr.cv - 2.0) * T;
@@ -132,12 +132,20 @@ __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1)
           }
       }
       const NodeState s = node_moments<P, BLOCK>(pr, cl, code, nb);
-      int n2 = NEWTON_UNREALIZABLE;
+      const NodeFields<P> nf = node_publish<P>(code, s, k, a.ps, a.mom_out, a.lat_out, a.nxt_out);
+      P first[NM];
+#pragma unroll
+      for (int j = 0; j < NM; ++j) first[j] = lam[j];
       bool fixed2 = false;
-      if (s.rho > 0.0)
-        n2 = node_equilibrium<P, BLOCK>(pr, cl, s.ubx, s.uby, s.T, pr.warm, lam, &cnt, &fixed2);
-      node_store<P, BLOCK>(pr, cl, code, s, n2, fixed2, pr.warm, lam, k, a.ps, a.pop_out, a.mom_out,
-                           a.lat_out, a.nxt_out, a.lam_out, &n_fail);
+      const int n2 = node_equilibrium<P, BLOCK>(
+          pr, cl, s, pr.warm,
+          [&](P* l) {
+#pragma unroll
+            for (int j = 0; j < NM; ++j) l[j] = first[j];
+          },
+          lam, &cnt, nullptr, &fixed2);
+      if (!node_store<P, BLOCK>(pr, cl, nf, n2, fixed2, pr.warm, lam, k, a.ps, a.pop_out, a.lam_out))
+        n_fail += 1;
     } else {
       for (int i = 0; i < NPLANES; ++i) a.pop_out[i * a.ps + k] = (P)0;
       a.mom_out[k] = (P)r;

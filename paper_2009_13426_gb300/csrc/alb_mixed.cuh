@@ -123,13 +123,14 @@ static_assert(XI_X(PX + 16) == 3 && XI_X(PX + 18) == -3 && XI_Y(PY + 8) == 2 &&
               "index pattern of the velocity groups");
 
 // 2^(j/N), j = 0..N-1 (N = EXPT_N); kernels copy it to shared memory (lanes
-// index it freely).
-static __constant__ double c_exptab[EXPT_N] = {ALB_EXPT_TABLE_VALUES};
+// index it freely). In global memory: consecutive threads copy consecutive
+// entries, which constant memory would serve one by one.
+static __device__ const double g_exptab[EXPT_N] = {ALB_EXPT_TABLE_VALUES};
 
 // Copy the table into a block's shared array of EXPT_N doubles (all threads;
 // includes a barrier).
 __device__ __forceinline__ void load_exptab(double* s_tab) {
-  for (int j = threadIdx.x; j < EXPT_N; j += blockDim.x) s_tab[j] = c_exptab[j];
+  for (int j = threadIdx.x; j < EXPT_N; j += blockDim.x) s_tab[j] = g_exptab[j];
   __syncthreads();
 }
 
@@ -711,7 +712,8 @@ __device__ __forceinline__ void shift_multipliers(const R l[NM], R dx, R dy, R o
 // between this phase and the refinement. What is live across a pass is kept
 // small for the same reason: the last step's direction and length but not its
 // start, and the three inputs instead of the eight targets. *gres is the
-// residual maximum (FP32) at the last evaluated point.
+// residual maximum (FP32) at the last evaluated point, *stale says that the
+// factor is of the point before the returned one.
 //
 // FACTOR = false is the prelude of the FP64 plain path: it stops, without a
 // factor, at the first point from which the predicted decrease of the dual lies
@@ -722,9 +724,11 @@ __device__ __forceinline__ void shift_multipliers(const R l[NM], R dx, R dy, R o
 // from the oracle by 1.1e-10 in 1000 steps where it stays below 1e-11 so.
 template <bool FACTOR>
 __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int maxit, bool warm,
-                                           float lam[NM], Fact32& fc, int* iters, float* gres) {
+                                           float lam[NM], Fact32& fc, int* iters, float* gres,
+                                           bool* stale) {
   enum { START_WARM, START_MAXWELL, TRIAL, RETURNED };
   *iters = 0;
+  *stale = false;
   // Maxwellian multipliers with lambda_0 = 0 (fixed from the normalisation
   // once evaluated)
   auto maxwell = [&]() {
@@ -822,6 +826,7 @@ __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int ma
       // by some 1e-3, so it still contracts by about that per residual, at
       // 0.6 more residuals a solve than with a fresh factor but without the
       // pass and the factorisation that one takes.
+      *stale = true;
       ++it;
       break;
     }
@@ -1229,8 +1234,9 @@ static __device__ __noinline__ int solve_mixed64(double ubx, double uby, double 
   for (int k = 0; k < NM; ++k) dl[k] = warm ? cvt_f32_rn(lam[k]) : 0.0f;
   for (bool w = warm;; w = false) {
     int it = 0;
+    bool stale;
     st = newton_fp32<false>(cvt_f32_rn(ubx), cvt_f32_rn(uby), cvt_f32_rn(T), 30, w, dl, fc, &it,
-                            &gres);
+                            &gres, &stale);
     *it32 += it;
     if (st == NEWTON_OK || !w) break;
   }
@@ -1429,6 +1435,54 @@ static __device__ __noinline__ int newton4_fp64g(double ubx, double uby, double 
   }
 }
 
+// The change of the constraint sums under a small step dl of the multipliers, sum
+// p_i (exp(-d_i) - 1) P(xi_i), in FP32 (in units of 2^-31): its relative error of
+// some 1e-7 lies far below what the step leaves.
+struct PassDelta {
+  float M[NM];
+  const uint64_t* col;
+  int stride;
+  __device__ __forceinline__ PassDelta(const uint64_t* c, int s) : col(c), stride(s) {
+#pragma unroll
+    for (int k = 0; k < NM; ++k) M[k] = 0.0f;
+  }
+  __device__ __forceinline__ float w(int i, float d) const {
+    const uint32_t hi = reinterpret_cast<const uint32_t*>(col)[2 * i * stride + 1];
+    return mul_rn((float)hi, mul_rn(d, fmaf(d, fmaf(d, -1.0f / 6.0f, 0.5f), -1.0f)));
+  }
+  __device__ __forceinline__ void rest(float d) { M[0] += w(0, d); }
+  template <int AX>
+  __device__ __forceinline__ void add_pair(const Pow<float>& k, float p, float m) {
+    const float S = p + m, D = p - m;
+    M[0] += S;
+    M[AX ? 2 : 1] = fmaf(k.a, D, M[AX ? 2 : 1]);
+    M[AX ? 5 : 3] = fmaf(k.a2, S, M[AX ? 5 : 3]);
+    M[AX ? 7 : 6] = fmaf(k.a3, D, M[AX ? 7 : 6]);
+  }
+  __device__ __forceinline__ void pair_x(int g, const Pow<float>& k, float dp, float dm) {
+    add_pair<0>(k, w(PX + 8 * g, dp), w(PX + 2 + 8 * g, dm));
+  }
+  __device__ __forceinline__ void pair_y(int g, const Pow<float>& k, float dp, float dm) {
+    add_pair<1>(k, w(PY + 8 * g, dp), w(PY + 2 + 8 * g, dm));
+  }
+  __device__ __forceinline__ void quad(int g, const Pow<float>& k, float dpp, float dmp, float dmm,
+                                       float dpm) {
+    const float ppp = w(PQ + 8 * g, dpp), pmp = w(PQ + 1 + 8 * g, dmp);
+    const float pmm = w(PQ + 2 + 8 * g, dmm), ppm = w(PQ + 3 + 8 * g, dpm);
+    const float Ap = ppp + ppm, Bm = pmp + pmm, Cp = ppp - ppm, Dm = pmp - pmm;
+    const float sum = Ap + Bm, xs = Ap - Bm, ys = Cp + Dm, xys = Cp - Dm;
+    const float t3 = k.a3 + k.a3;
+    M[0] += sum;
+    M[1] = fmaf(k.a, xs, M[1]);
+    M[2] = fmaf(k.a, ys, M[2]);
+    M[3] = fmaf(k.a2, sum, M[3]);
+    M[4] = fmaf(k.a2, xys, M[4]);
+    M[5] = fmaf(k.a2, sum, M[5]);
+    M[6] = fmaf(t3, xs, M[6]);
+    M[7] = fmaf(t3, ys, M[7]);
+  }
+};
+
 // Largest exponent |1 + lambda . P(xi_i)| over the velocities is at most this:
 // the larger of the axis and the diagonal velocities' bounds.
 __device__ __forceinline__ float exponent_bound(const float l[NM]) {
@@ -1448,7 +1502,7 @@ __device__ __forceinline__ float exponent_bound(const float l[NM]) {
 // 1/64: the Q63 residual has to stay below one) and for failures; the caller
 // then refines in FP64.
 __device__ __forceinline__ int refine_fix(double ubx, double uby, double T, float tolf, int maxr,
-                                          float lam[NM], const Fact32& fc, float gres,
+                                          float lam[NM], const Fact32& fc, float gres, bool stale,
                                           const uint64_t* tab, uint64_t* col, int stride,
                                           int* evals, int* updates) {
   *evals = 0;
@@ -1492,37 +1546,55 @@ __device__ __forceinline__ int refine_fix(double ubx, double uby, double T, floa
     if (r >= maxr) return NEWTON_MAXIT;
     solve32(fc, g32, dl);
     bound = step_exponent_bound(dl);  // (a NaN fails both comparisons)
+    if (r == 0 && stale && bound <= FIX_STEP_MAX) {
+      // With the factor one step old, this step leaves some 1e-3 of the
+      // residual: 1e-10, for a second update. What it leaves is known in FP32
+      // from the change of the sums, and a second correction joins the step
+      // before the column is updated once (250 operations instead of a pass of
+      // some 700).
+      PassDelta pd(col, stride);
+      visit_speeds<float>(dl, pd, 0.0f);
+      float d2[NM];
+#pragma unroll
+      for (int k = 0; k < NM; ++k) g32[k] = fmaf(pd.M[k], 4.656612873077393e-10f, g32[k]);
+      solve32(fc, g32, d2);
+#pragma unroll
+      for (int k = 0; k < NM; ++k) dl[k] += d2[k];
+      bound = step_exponent_bound(dl);
+    }
 #pragma unroll
     for (int k = 0; k < NM; ++k) lam[k] += dl[k];
   }
 }
 
+constexpr int WORK_EVALS = 12, WORK_UPDATES = 22;
+
 // FP32 Newton from the warm start if given, else (or if that fails) from the
 // Maxwellian, then the fixed-point refinement: on NEWTON_OK the Q63 column and
-// the multipliers in lam.
+// the multipliers in lam. *work collects the counts of a node's solves in one
+// register: FP32 steps (at most 62 a solve), evaluations and updates (at most 7)
+// in 12, 10 and 10 bits, enough for the 23 solves of a thread and tile.
 //
 // lam holds the warm start on entry if `warm` is set. Inlined: a call would save
 // and restore some sixty registers per thread through local memory, which
 // at two blocks of columns per SM leaves L1.
 __device__ __forceinline__ int solve_fix(double ubx, double uby, double T, float tolf, bool warm,
                                          const uint64_t* ftab, uint64_t* col, int stride,
-                                         float lam[NM], SolveCount* cnt) {
+                                         float lam[NM], unsigned* work) {
   const float ubx32 = cvt_f32_rn(ubx), uby32 = cvt_f32_rn(uby), T32 = cvt_f32_rn(T);
   Fact32 fc;
   float gres = 0.0f;
-  int st;
+  bool stale = false;
+  int st, it = 0, ev = 0, up = 0;
   for (bool w = warm;; w = false) {
     int it32 = 0;
-    st = newton_fp32<true>(ubx32, uby32, T32, 30, w, lam, fc, &it32, &gres);
-    cnt->fp32_iters += it32;
+    st = newton_fp32<true>(ubx32, uby32, T32, 30, w, lam, fc, &it32, &gres, &stale);
+    it += it32;
     if (st == NEWTON_OK || !w) break;
   }
-  if (st == NEWTON_OK) {
-    int ev = 0, up = 0;
-    st = refine_fix(ubx, uby, T, tolf, 6, lam, fc, gres, ftab, col, stride, &ev, &up);
-    cnt->fp64_evals += ev;
-    cnt->fp64_updates += up;
-  }
+  if (st == NEWTON_OK)
+    st = refine_fix(ubx, uby, T, tolf, 6, lam, fc, gres, stale, ftab, col, stride, &ev, &up);
+  *work += (unsigned)it + ((unsigned)ev << WORK_EVALS) + ((unsigned)up << WORK_UPDATES);
   return st;
 }
 
@@ -1723,7 +1795,8 @@ static __device__ __noinline__ int equilibrium_mixed(double ubx, double uby, dou
     for (int k = 0; k < NM; ++k) l32[k] = warm[k];
   for (;;) {
     int it32 = 0;
-    st = newton_fp32<true>(ubx32, uby32, T32, 30, w, l32, fc, &it32, &gres);
+    bool stale;
+    st = newton_fp32<true>(ubx32, uby32, T32, 30, w, l32, fc, &it32, &gres, &stale);
     cnt->fp32_iters += it32;
     if (st == NEWTON_OK || !w) break;
     w = false;

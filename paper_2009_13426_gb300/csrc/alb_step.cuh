@@ -17,11 +17,12 @@ namespace alb {
 
 constexpr int BLOCK = 128;
 
-// Dynamic shared memory of a block: the fixed-point exponential's table (FP32
-// form), then the two columns of every thread.
+// Dynamic shared memory of a block: the tables of the exponentials (FP64, and
+// fixed-point in the FP32 form), then the two columns of every thread.
 template <typename P>
 constexpr size_t table_bytes() {
-  return std::is_same<P, float>::value ? FIXT_N * sizeof(uint64_t) : 0;
+  return EXPT_N * sizeof(double) +
+         (std::is_same<P, float>::value ? FIXT_N * sizeof(uint64_t) : 0);
 }
 template <typename P, int B = BLOCK>
 constexpr size_t smem_bytes() {
@@ -36,121 +37,185 @@ struct Columns {
   double* eq;
   const uint64_t* fixtab;
   const double* exptab;
-  // All threads of the block construct it (load_exptab includes a barrier);
-  // s_exptab: EXPT_N doubles of shared memory.
-  __device__ __forceinline__ Columns(unsigned char* smem, double* s_exptab) {
-    if constexpr (std::is_same<P, float>::value) load_fixtab(reinterpret_cast<uint64_t*>(smem));
-    load_exptab(s_exptab);
-    fixtab = reinterpret_cast<const uint64_t*>(smem);
-    exptab = s_exptab;
+  // All threads of the block construct it (it includes a barrier).
+  __device__ __forceinline__ explicit Columns(unsigned char* smem) {
+    fixtab = reinterpret_cast<const uint64_t*>(smem + EXPT_N * sizeof(double));
+    exptab = reinterpret_cast<const double*>(smem);
+    if constexpr (std::is_same<P, float>::value) load_fixtab(const_cast<uint64_t*>(fixtab));
+    load_exptab(const_cast<double*>(exptab));
     pop = reinterpret_cast<P*>(smem + table_bytes<P>()) + threadIdx.x;
     eq = reinterpret_cast<double*>(smem + table_bytes<P>() + (size_t)NPLANES * B * sizeof(P)) +
          threadIdx.x;
   }
 };
 
-// Equilibrium of one node in the storage precision P: FP32 Newton steps and FP64
-// residuals for the FP64 plain path (or all FP64 steps: Params::mixed64), FP32 Newton with the fixed-point refinement for the FP32
-// form (FP64 refinement where that does not reach), both started from the
-// multipliers in lam (precision P) if `warm` is set. The equilibrium per unit
-// density lands in the thread's column (Q63 instead of FP64 where *fixed is
-// set), the multipliers (in the precision P the warm start keeps them in) in
-// lam; after a failure lam is the warm start again.
-template <typename P, int B>
-__device__ __forceinline__ int node_equilibrium(const Params& pr, const Columns<P, B>& cl,
-                                                double ubx, double uby, double T, bool warm,
-                                                P lam[NM], SolveCount* cnt, bool* fixed) {
-  *fixed = false;
-  if (!(T > 0.0) || !isfinite(T) || !isfinite(ubx) || !isfinite(uby)) return NEWTON_UNREALIZABLE;
-  P w[NM];
-#pragma unroll
-  for (int k = 0; k < NM; ++k) w[k] = lam[k];
+// A node: density, velocity in the lattice frame, temperature, next lattice.
+struct NodeState {
+  double rho, ubx, uby, T;
+  int code2;
+};
+
+// A solve as handed to the function that is not inlined. What the caller keeps
+// across that call is kept small: values live across a call are spilled around it
+// on every path, also where the call is not taken.
+struct SolveIO {
+  double ubx, uby, T;
+  float lam[NM];
+  bool warm, fixed;
+};
+
+// Counts of a solve, added to the flow's counters by the lanes that made one.
+__device__ __forceinline__ void lanes_count(unsigned long long* ctr, unsigned v) {
+  const unsigned m = __activemask();
+  const unsigned sum = __reduce_add_sync(m, v);
+  if ((int)(threadIdx.x & 31) == __ffs(m) - 1 && sum) atomicAdd(ctr, (unsigned long long)sum);
+}
+
+// Solves of the FP32 form outside its inlined path: the reduced model, and the
+// states the fixed-point refinement does not take.
+template <int B>
+static __device__ __noinline__ int solve_other(const Params& pr, const double* exptab,
+                                               const uint64_t* fixtab, double* eq, SolveIO* io,
+                                               unsigned long long* ctr) {
+  const double ubx = io->ubx, uby = io->uby, T = io->T;
+  const bool warm = io->warm;
+  float lam[NM];
+  SolveCount cnt;
   int st;
+#pragma unroll
+  for (int k = 0; k < NM; ++k) lam[k] = io->lam[k];
+  io->fixed = false;
   if (pr.moments == 4) {
-    // reduced model: in the FP32 form as the full one, else (and where that
-    // does not reach) an FP64 4x4 Newton
-    int it = 0, ev = 0;
-    st = NEWTON_SINGULAR;
-    if constexpr (std::is_same<P, float>::value) {
-      int it32 = 0, up = 0;
-      float l32[NM];
-#pragma unroll
-      for (int k = 0; k < NM; ++k) l32[k] = lam[k];
-      st = solve4_fix(ubx, uby, T, (float)pr.tol, warm, cl.fixtab,
-                      reinterpret_cast<uint64_t*>(cl.eq), B, l32, &it32, &ev, &up);
-      cnt->fp32_iters += it32;
-      cnt->fp64_evals += ev;
-      cnt->fp64_updates += up;
-      *fixed = st == NEWTON_OK;
-      if (st == NEWTON_OK)
-#pragma unroll
-        for (int k = 0; k < NM; ++k) lam[k] = l32[k];
-    }
+    int it32 = 0, ev = 0, up = 0;
+    st = solve4_fix(ubx, uby, T, (float)pr.tol, warm, fixtab, reinterpret_cast<uint64_t*>(eq), B,
+                    lam, &it32, &ev, &up);
+    cnt.fp32_iters = it32;
+    cnt.fp64_evals = ev;
+    cnt.fp64_updates = up;
+    io->fixed = st == NEWTON_OK;
     if (st != NEWTON_OK) {
       double w8[NM], l8[NM];
+      int it = 0;
 #pragma unroll
-      for (int k = 0; k < NM; ++k) w8[k] = warm ? (double)lam[k] : 0.0;
-      st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l8, &it, &ev,
+      for (int k = 0; k < NM; ++k) w8[k] = warm ? (double)io->lam[k] : 0.0;
+      st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, exptab, eq, B, l8, &it, &ev,
                          warm ? w8 : nullptr);
-      cnt->fp64_iters += it;
-      cnt->fp64_evals += ev;
+      cnt.fp64_iters += it;
+      cnt.fp64_evals += ev;
       if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
-        st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l8, &it, &ev,
-                           nullptr);
-        cnt->fp64_iters += it;
-        cnt->fp64_evals += ev;
+        st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, exptab, eq, B, l8, &it, &ev, nullptr);
+        cnt.fp64_iters += it;
+        cnt.fp64_evals += ev;
       }
 #pragma unroll
-      for (int k = 0; k < NM; ++k) lam[k] = (P)l8[k];
-    }
-  } else if constexpr (std::is_same<P, float>::value) {
-    st = solve_fix(ubx, uby, T, (float)pr.tol, warm, cl.fixtab, reinterpret_cast<uint64_t*>(cl.eq),
-                   B, lam, cnt);
-    *fixed = st == NEWTON_OK;
-    if (st != NEWTON_OK) {
-      SolveCount c;  // of its own: the callers' counts stay in registers
-      float l32[NM];
-#pragma unroll
-      for (int k = 0; k < NM; ++k) l32[k] = w[k];
-      st = equilibrium_mixed(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, warm ? l32 : nullptr, cl.eq,
-                             B, l32, nullptr, &c);
-      cnt->add(c);
-#pragma unroll
-      for (int k = 0; k < NM; ++k) lam[k] = l32[k];
+      for (int k = 0; k < NM; ++k) lam[k] = (float)l8[k];
     }
   } else {
-    int it = 0, ev = 0;
-    double l64[NM];
-    st = NEWTON_SINGULAR;
-    if (pr.mixed64) {
-      int it32 = 0;
+    st = equilibrium_mixed(ubx, uby, T, pr.tol, pr.maxit, exptab, warm ? io->lam : nullptr, eq, B,
+                           lam, nullptr, &cnt);
+  }
+  if (ctr) {
+    lanes_count(ctr + CTR_FP32_ITERS, cnt.fp32_iters);
+    lanes_count(ctr + CTR_NEWTON_ITERS, cnt.fp64_iters);
+    lanes_count(ctr + CTR_FP64_EVALS, cnt.fp64_evals);
+    lanes_count(ctr + CTR_FP64_UPDATES, cnt.fp64_updates);
+  }
+  if (st == NEWTON_OK)
 #pragma unroll
-      for (int k = 0; k < NM; ++k) l64[k] = lam[k];
-      st = solve_mixed64(ubx, uby, T, pr.tol, warm, cl.exptab, cl.eq, B, l64, &it32, &it, &ev);
-      cnt->fp32_iters += it32;
-      cnt->fp64_iters += it32 + it;
-      cnt->fp64_evals += ev;
+    for (int k = 0; k < NM; ++k) io->lam[k] = lam[k];
+  return st;
+}
+
+// Counts of one node update, added to the flow's counters warp by warp.
+template <typename P>
+struct NodeCount {
+  unsigned n = 0;    // rebuilt pulls (10 bits), those that fell back (10), solves (11), failed (1)
+  unsigned fix = 0;  // FP32 form: counts of solve_fix
+  SolveCount solve;  // FP64 plain
+};
+constexpr unsigned N_REC = 1u, N_REC_FAIL = 1u << 10, N_CALLS = 1u << 20, N_FAIL = 1u << 31;
+
+// Equilibrium of one node in the storage precision P: FP32 Newton steps and FP64
+// residuals for the FP64 plain path (or all FP64 steps: Params::mixed64), FP32
+// Newton with the fixed-point refinement for the FP32 form (solve_other where
+// that does not reach). If `warm` is set, both start from the multipliers that
+// load(lam) gives. The equilibrium per unit density lands in the thread's column
+// (Q63 instead of FP64 where *fixed is set), the multipliers (in the precision P
+// the warm start keeps them in) in lam; after a failure lam is the warm start
+// again. ctr (or null) counts the solves of solve_other.
+template <typename P, int B, typename Load>
+__device__ __forceinline__ int node_equilibrium(const Params& pr, const Columns<P, B>& cl,
+                                                const NodeState& s, bool warm, Load load, P lam[NM],
+                                                NodeCount<P>* nc, unsigned long long* ctr,
+                                                bool* fixed) {
+  *fixed = false;
+  const double ubx = s.ubx, uby = s.uby, T = s.T;
+  if (warm) load(lam);
+  if (!(s.rho > 0.0) || !(T > 0.0) || !isfinite(T) || !isfinite(ubx) || !isfinite(uby))
+    return NEWTON_UNREALIZABLE;
+  if constexpr (std::is_same<P, float>::value) {
+    int st = NEWTON_SINGULAR;
+    if (pr.moments == 8)
+      st = solve_fix(ubx, uby, T, (float)pr.tol, warm, cl.fixtab,
+                     reinterpret_cast<uint64_t*>(cl.eq), B, lam, &nc->fix);
+    *fixed = st == NEWTON_OK;
+    if (st != NEWTON_OK) {
+      SolveIO io;
+      io.ubx = ubx;
+      io.uby = uby;
+      io.T = T;
+      io.warm = warm;
+      if (warm) load(io.lam);
+      st = solve_other<B>(pr, cl.exptab, cl.fixtab, cl.eq, &io, ctr);
+      *fixed = io.fixed;
+#pragma unroll
+      for (int k = 0; k < NM; ++k) lam[k] = io.lam[k];
+    }
+    return st;
+  } else {
+    int it = 0, ev = 0, st = NEWTON_SINGULAR;
+    double w[NM];
+#pragma unroll
+    for (int k = 0; k < NM; ++k) w[k] = lam[k];
+    if (pr.moments == 4) {
+      st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, lam, &it, &ev,
+                         warm ? w : nullptr);
+      nc->solve.fp64_iters += it;
+      nc->solve.fp64_evals += ev;
+      if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
+        st = newton4_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, lam, &it, &ev,
+                           nullptr);
+        nc->solve.fp64_iters += it;
+        nc->solve.fp64_evals += ev;
+      }
+    } else {
+      if (pr.mixed64) {
+        int it32 = 0;
+        st = solve_mixed64(ubx, uby, T, pr.tol, warm, cl.exptab, cl.eq, B, lam, &it32, &it, &ev);
+        nc->solve.fp32_iters += it32;
+        nc->solve.fp64_iters += it32 + it;
+        nc->solve.fp64_evals += ev;
+      }
+      if (st != NEWTON_OK) {
+        st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, lam, &it, &ev,
+                          warm ? w : nullptr);
+        nc->solve.fp64_iters += it;
+        nc->solve.fp64_evals += ev;
+      }
+      if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
+        // the previous multipliers led nowhere: start again from the Maxwellian
+        st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, lam, &it, &ev,
+                          nullptr);
+        nc->solve.fp64_iters += it;
+        nc->solve.fp64_evals += ev;
+      }
     }
     if (st != NEWTON_OK) {
-      st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l64, &it, &ev,
-                        warm ? w : nullptr);
-      cnt->fp64_iters += it;
-      cnt->fp64_evals += ev;
-    }
-    if (warm && st != NEWTON_OK && st != NEWTON_UNREALIZABLE) {
-      // the previous multipliers led nowhere: start again from the Maxwellian
-      st = newton_fp64g(ubx, uby, T, pr.tol, pr.maxit, cl.exptab, cl.eq, B, l64, &it, &ev, nullptr);
-      cnt->fp64_iters += it;
-      cnt->fp64_evals += ev;
-    }
 #pragma unroll
-    for (int k = 0; k < NM; ++k) lam[k] = l64[k];
+      for (int k = 0; k < NM; ++k) lam[k] = w[k];
+    }
+    return st;
   }
-  if (st != NEWTON_OK) {
-#pragma unroll
-    for (int k = 0; k < NM; ++k) lam[k] = w[k];
-  }
-  return st;
 }
 
 // Moment accumulation: plain in FP64; Neumaier-compensated in FP32.
@@ -308,6 +373,13 @@ __device__ __forceinline__ float rel_dev(float f, float fe) {
 }
 __device__ __forceinline__ double rel_dev(double f, double fe) { return fabs(f - fe) / fe; }
 
+// What the collision needs of a node's moments, in the population precision: the
+// velocity (bx, by) in the lattice frame is that of the rounded absolute one.
+template <typename P>
+struct NodeFields {
+  P rho, T, bx, by;
+};
+
 // Store of a collided node for Pr != 1: BGK plus the heat-flux term of App. E
 // (Eqs. Shakhov, prandtlPoly),
 //   f* += (1/tau - 1/tau_Pr) q.cbar / (rho Cp T^2) (|cbar|^2 / (2T) - Cp) f^eq,
@@ -318,11 +390,9 @@ __device__ __forceinline__ double rel_dev(double f, double fe) { return fabs(f -
 // sensor factor tau / (1/2 + nu/T).
 template <typename P, int B>
 __device__ __forceinline__ void store_shakhov(const Params& pr, const P* st, const P* eqv,
-                                              double rho, double ux, double uy, double T,
-                                              int code, P tau, size_t k, size_t ps,
-                                              P* __restrict__ pop_out) {
-  const P Tp = (P)T, rp = (P)rho;
-  const P bx = (P)(ux - (double)lat_ux(code)), by = (P)(uy - (double)lat_uy(code));
+                                              const NodeFields<P>& nf, P tau, size_t k,
+                                              size_t ps, P* __restrict__ pop_out) {
+  const P Tp = nf.T, rp = nf.rho, bx = nf.bx, by = nf.by;
   const P cp = (P)pr.cp;
   const P gp = mul_rn(fma((P)2, (P)pr.cv, (P)-2), Tp);
   const P tau_pr = mul_rn((P)0.5 + (P)pr.kappa_nu / Tp, tau / ((P)0.5 + (P)pr.nu / Tp));
@@ -359,10 +429,6 @@ __device__ __forceinline__ void store_shakhov(const Params& pr, const P* st, con
 
 // Moments of one node whose 42 pre-collision populations sit in its shared
 // column, and the lattice of its next pull.
-struct NodeState {
-  double rho, ubx, uby, T;  // density, velocity in the lattice frame, temperature
-  int code2;                // next lattice
-};
 template <typename P, int B>
 __device__ __forceinline__ NodeState node_moments(const Params& pr, const Columns<P, B>& cl,
                                                   int code, const uint8_t* nb) {
@@ -408,20 +474,35 @@ __device__ __forceinline__ NodeState node_moments(const Params& pr, const Column
   return NodeState{rho, ubx, uby, T, code2};
 }
 
+// Stores a node's moments and lattices; done before the solve, so that little
+// of the node is live across it.
+template <typename P>
+__device__ __forceinline__ NodeFields<P> node_publish(int code, const NodeState& s, size_t k,
+                                                      size_t ps, P* __restrict__ mom_out,
+                                                      uint8_t* lat_out, uint8_t* nxt_out) {
+  const double Ux = cvt_f64(lat_ux(code)), Uy = cvt_f64(lat_uy(code));
+  const double ux = s.ubx + Ux, uy = s.uby + Uy;
+  const NodeFields<P> f{to_p<P>(s.rho), to_p<P>(s.T), to_p<P>(ux - Ux), to_p<P>(uy - Uy)};
+  mom_out[k] = f.rho;
+  mom_out[ps + k] = to_p<P>(ux);
+  mom_out[2 * ps + k] = to_p<P>(uy);
+  mom_out[3 * ps + k] = f.T;
+  lat_out[k] = (uint8_t)code;
+  nxt_out[k] = (uint8_t)s.code2;
+  return f;
+}
+
 // Collision of a node (BGK, or App. E for Pr != 1) with the equilibrium in its
 // column (solve status ns, multipliers lam: the warm start's after a failure),
-// then the store of its state. A failed node is left uncollided and counted.
+// then the store of its populations and multipliers. Returns false if the solve
+// failed: the node is then left uncollided.
 template <typename P, int B>
-__device__ __forceinline__ void node_store(const Params& pr, const Columns<P, B>& cl, int code,
-                                           const NodeState& s, int ns, bool fixed, bool warm,
+__device__ __forceinline__ bool node_store(const Params& pr, const Columns<P, B>& cl,
+                                           const NodeFields<P>& nf, int ns, bool fixed, bool warm,
                                            const P lam[NM], size_t k, size_t ps,
-                                           P* __restrict__ pop_out, P* __restrict__ mom_out,
-                                           uint8_t* lat_out, uint8_t* nxt_out, P* lam_out,
-                                           unsigned* n_fail) {
+                                           P* __restrict__ pop_out, P* lam_out) {
   const P* st = cl.pop;
-  const double rho = s.rho, T = s.T;
-  const double ux = s.ubx + cvt_f64(lat_ux(code)), uy = s.uby + cvt_f64(lat_uy(code));
-  // multipliers for the next step's warm start (lattice `code`), if stored
+  // multipliers for the next step's warm start, if stored
   if (lam_out) {
 #pragma unroll
     for (int j = 0; j < NM; ++j)
@@ -431,10 +512,9 @@ __device__ __forceinline__ void node_store(const Params& pr, const Columns<P, B>
   if (ns == NEWTON_OK) {
     // f^eq = rho p, g^eq = (2 Cv - D) T f^eq and tau = 1/2 + nu/T in the
     // population precision (in the FP32 form from the FP64 equilibrium)
-    const P Tp = to_p<P>(T);
+    const P Tp = nf.T, rp = nf.rho;
     const P gp = mul_rn(fma((P)2, to_p<P>(pr.cv), (P)-2), Tp);
     P tau = (P)0.5 + to_p<P>(pr.nu) / Tp;
-    const P rp = to_p<P>(rho);
     const P* eqv = eq_in_precision<P, B>(cl.eq, fixed);
     constexpr int es = eq_stride<P, B>();
     if (pr.sensor) {
@@ -448,7 +528,7 @@ __device__ __forceinline__ void node_store(const Params& pr, const Columns<P, B>
       tau = mul_rn(tau, sensor_alpha<P>(pr, eps));
     }
     if (pr.shakhov) {
-      store_shakhov<P, B>(pr, st, eqv, rho, ux, uy, T, code, tau, k, ps, pop_out);
+      store_shakhov<P, B>(pr, st, eqv, nf, tau, k, ps, pop_out);
     } else {
       const P om = (P)1 / tau;
 #pragma unroll
@@ -461,17 +541,11 @@ __device__ __forceinline__ void node_store(const Params& pr, const Columns<P, B>
         __stcs(&pop_out[(Q + i) * ps + k], fma(om, ge - g, g));
       }
     }
-  } else {
-    *n_fail += 1;
-#pragma unroll
-    for (int i = 0; i < NPLANES; ++i) pop_out[i * ps + k] = st[i * B];
+    return true;
   }
-  mom_out[k] = to_p<P>(rho);
-  mom_out[ps + k] = to_p<P>(ux);
-  mom_out[2 * ps + k] = to_p<P>(uy);
-  mom_out[3 * ps + k] = to_p<P>(T);
-  lat_out[k] = (uint8_t)code;
-  nxt_out[k] = (uint8_t)s.code2;
+#pragma unroll
+  for (int i = 0; i < NPLANES; ++i) pop_out[i * ps + k] = st[i * B];
+  return false;
 }
 
 // Current lattices of the eight nodes around (x, y) (boundary rule for
@@ -491,49 +565,66 @@ __device__ __forceinline__ void neighbour_codes(const Params& pr, const uint8_t*
     }
 }
 
-// Counts of one node update, added to the flow's counters warp by warp.
-struct NodeCount {
-  SolveCount solve;
-  unsigned rec = 0, rec_fail = 0, fail = 0, calls = 0;
-};
-
-__device__ __forceinline__ void flush_counts(unsigned long long* ctr, const NodeCount& c) {
-  warp_count(ctr + CTR_NEWTON_ITERS, c.solve.fp64_iters);
-  warp_count(ctr + CTR_FP64_EVALS, c.solve.fp64_evals);
-  warp_count(ctr + CTR_FP32_ITERS, c.solve.fp32_iters);
-  warp_count(ctr + CTR_FP64_UPDATES, c.solve.fp64_updates);
-  warp_count(ctr + CTR_NEWTON_CALLS, c.calls);
-  warp_count(ctr + CTR_NEWTON_FAIL, c.fail);
-  warp_count(ctr + CTR_REC, c.rec);
-  warp_count(ctr + CTR_REC_FAIL, c.rec_fail);
+template <typename P>
+__device__ __forceinline__ void flush_counts(unsigned long long* ctr, const NodeCount<P>& c) {
+  if constexpr (std::is_same<P, float>::value) {
+    warp_count(ctr + CTR_FP32_ITERS, c.fix & ((1u << WORK_EVALS) - 1u));
+    warp_count(ctr + CTR_FP64_EVALS, (c.fix >> WORK_EVALS) & 1023u);
+    warp_count(ctr + CTR_FP64_UPDATES, c.fix >> WORK_UPDATES);
+  } else {
+    warp_count(ctr + CTR_NEWTON_ITERS, c.solve.fp64_iters);
+    warp_count(ctr + CTR_FP64_EVALS, c.solve.fp64_evals);
+    warp_count(ctr + CTR_FP32_ITERS, c.solve.fp32_iters);
+    warp_count(ctr + CTR_FP64_UPDATES, c.solve.fp64_updates);
+  }
+  warp_count(ctr + CTR_NEWTON_CALLS, (c.n >> 20) & 2047u);
+  warp_count(ctr + CTR_NEWTON_FAIL, c.n >> 31);
+  warp_count(ctr + CTR_REC, c.n & 1023u);
+  warp_count(ctr + CTR_REC_FAIL, (c.n >> 10) & 1023u);
 }
 
-// Shared state of a block's rebuilds: one entry (owner thread << 5 | i) per
-// missing pull of the block's nodes, at most Q per node. They are handled in
-// chunks of CHUNK entries; within a chunk, every distinct (sender, receiver
-// lattice) is entered once into a hash table and solved once.
-template <int B>
+// Shared state of a block's rebuilds. The missing pulls are numbered in (thread,
+// velocity) order by a prefix sum of the threads' counts and handled in chunks of
+// CHUNK; an entry is found again from its number (the thread by bisection, the
+// velocity from the thread's mask). Within a chunk, every distinct (sender,
+// receiver lattice) is entered once into a hash table and solved once. The table
+// keeps key and solve in one word: with these sizes two blocks of the FP32 form
+// leave 60 KB of an SM to L1, where their stack lives (28 KB with a list of the
+// entries and separate arrays).
+template <typename P, int B>
 struct RebuildQueue {
-  static constexpr int PER = 3;          // entries per thread and chunk
+  static constexpr bool LARGE = std::is_same<P, float>::value && B > 128;
+  static constexpr int PER = LARGE ? 2 : 3;        // entries per thread and chunk
   static constexpr int CHUNK = PER * B;
-  static constexpr int HASH = 4 * B;     // positions (a power of two), at most 3/4 used
-  static constexpr int SHIFT = B == 32 ? 25 : B == 64 ? 24 : B == 128 ? 23 : 22;  // 32 - log2(HASH)
-  static_assert(HASH == 1 << (32 - SHIFT), "hash positions");
-  unsigned short entry[Q * B];
-  unsigned hkey[HASH];          // key of a position, or EMPTY
-  unsigned short hslot[HASH];   // its solve
-  unsigned skey[CHUNK];         // key of each solve
+  static constexpr int HASH = (LARGE ? 3 : 4) * B; // positions: at most 3/4 used
+  static constexpr int KEY_BITS = 20;
+  static_assert(CHUNK < 1 << (32 - KEY_BITS), "solve numbers");
+  unsigned hash[HASH];          // key (20 bits) and solve (12 bits) of a position, or EMPTY
+  unsigned short spos[CHUNK];   // position of each solve
+  unsigned miss[B];             // velocities missing at each thread's node
+  unsigned short start[B];      // number of the thread's first entry
   unsigned char state[B];       // of the solves of a round: 1 failed, 2 column in Q63
   int wsum[B / 32];             // missing pulls per warp
   int count, nsolve;
-};
-constexpr unsigned RB_EMPTY = 0xffffffffu;
 
-// Key of a rebuild solve: receiver lattice and sender position in the tile's
-// frame. The sender lies within 6 nodes of the tile (|xi| <= 3, |U| <= 3) and
-// the tile's sides are at most B <= 1000: 10 bits per coordinate.
-__device__ __forceinline__ unsigned rebuild_key(int code, int sx, int sy) {
-  return ((unsigned)code << 20) | ((unsigned)(sy + 8) << 10) | (unsigned)(sx + 8);
+  // Thread (upper bits) and velocity (5 bits) of entry e.
+  __device__ __forceinline__ unsigned entry(int e) const {
+    int o = 0;
+#pragma unroll
+    for (int d = B / 2; d > 0; d >>= 1)
+      if (start[o + d] <= e) o += d;
+    unsigned m = miss[o];
+    for (int j = e - start[o]; j > 0; --j) m &= m - 1;
+    return (unsigned)o << 5 | (unsigned)(__ffs(m) - 1);
+  }
+};
+constexpr unsigned RB_EMPTY = 0xffffffffu, RB_KEY = (1u << 20) - 1u;
+
+// Key of a rebuild solve: receiver lattice (below 49) and sender position in the
+// frame of a tile of 2^lg by B >> lg nodes. The sender lies within 6 nodes of the
+// tile (|xi| <= 3, |U| <= 3); 49 (2^lg + 16) ((B >> lg) + 16) stays below 2^18.
+__device__ __forceinline__ unsigned rebuild_key(int code, int sx, int sy, int lg) {
+  return (unsigned)code + 49u * (unsigned)(sx + 8 + (sy + 8) * ((1 << lg) + 16));
 }
 
 // Asynchronous copy of one population from global into shared memory, evicted
@@ -611,8 +702,8 @@ __device__ __forceinline__ unsigned pull_node(const StepArgs<P>& a, const Column
 // must call this (it holds barriers).
 template <typename P, int B>
 __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, int lg,
-                                          const Columns<P, B>& cl, RebuildQueue<B>& rq,
-                                          NodeCount& nc) {
+                                          const Columns<P, B>& cl, RebuildQueue<P, B>& rq,
+                                          NodeCount<P>& nc) {
   const Params& pr = a.prm;
   const size_t ps = a.ps;
   const int t = threadIdx.x;
@@ -631,10 +722,9 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
     own = pull_node<P, B>(a, cl, x, y, code, Upx, Upy, inside);
   }
   async_copies_wait();
-  // The queue of missing pulls in (thread, velocity) order, placed by a
-  // block-wide prefix sum of the threads' counts, so that its order, and with
-  // it which pulls share a solve below, does not depend on scheduling. A tile
-  // without missing pulls passes one barrier and skips the rest.
+  // Number the missing pulls: a block-wide prefix sum of the threads' counts, so
+  // that their order does not depend on scheduling. A tile without missing pulls
+  // passes one barrier and skips the rest.
   int nq = 0;
   {
     const unsigned miss = active ? (~own & ((1u << Q) - 1u)) : 0u;
@@ -647,11 +737,11 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
     }
     if (lane == 31) rq.wsum[warp] = incl;
     if (__syncthreads_or(nmiss)) {
-      int pos = incl - nmiss;
-      for (int w = 0; w < warp; ++w) pos += rq.wsum[w];
-      for (unsigned m = miss; m; m &= m - 1)
-        rq.entry[pos++] = (unsigned short)((t << 5) | (__ffs(m) - 1));
-      if (t == B - 1) rq.count = pos;  // the last thread's end: the total
+      int end = incl;
+      for (int w = 0; w < warp; ++w) end += rq.wsum[w];
+      rq.miss[t] = miss;
+      rq.start[t] = (unsigned short)(end - nmiss);
+      if (t == B - 1) rq.count = end;
       __syncthreads();
       nq = rq.count;
     }
@@ -661,63 +751,67 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
   // run B at a time in the columns of threads 0, 1, ...; every entry then takes
   // its value from the column of its solve (which entry comes first into the
   // table, and which thread solves it, changes no value).
-  static_assert(B % 32 == 0 && B <= 1000, "whole warps; tile sides fit the keys' 10-bit fields");
-  using RQ = RebuildQueue<B>;
+  static_assert(B % 32 == 0 && B <= 256, "whole warps; 13 bits for an entry");
+  using RQ = RebuildQueue<P, B>;
   P* const pop0 = cl.pop - t;  // column 0 of the block
   int base = 0, round = 0, nsolve = 0;  // chunk, its solves done, its solves
-  unsigned short pos[RQ::PER];          // hash position of this thread's entries
+  unsigned ent[RQ::PER];                // this thread's entries: hash position << 16 | entry
 #pragma unroll 1
   for (;;) {
     const bool rebuild = base < nq;
     if (rebuild && round == 0) {
-      for (int j = t; j < RQ::HASH; j += B) rq.hkey[j] = RB_EMPTY;
+      for (int j = t; j < RQ::HASH; j += B) rq.hash[j] = RB_EMPTY;
       if (t == 0) rq.nsolve = 0;
       __syncthreads();
 #pragma unroll
       for (int j = 0; j < RQ::PER; ++j) {
         const int e = base + j * B + t;
-        pos[j] = 0;
+        ent[j] = 0;
         if (e >= nq) continue;
-        const int owner = rq.entry[e] >> 5, i = rq.entry[e] & 31;
+        const unsigned en = rq.entry(e);
+        const int owner = en >> 5, i = en & 31;
         const int ox = owner & mask, oy = owner >> lg;
         const int oc = a.nxt_in[(size_t)(y0 + oy) * pr.nx + (x0 + ox)];
         const unsigned key =
-            rebuild_key(oc, ox - c_xi[i][0] - lat_ux(oc), oy - c_xi[i][1] - lat_uy(oc));
-        unsigned h = (key * 2654435761u) >> RQ::SHIFT;  // Knuth's multiplicative hash
-        for (;; h = (h + 1) % RQ::HASH) {
-          const unsigned old = atomicCAS(&rq.hkey[h], RB_EMPTY, key);
+            rebuild_key(oc, ox - c_xi[i][0] - lat_ux(oc), oy - c_xi[i][1] - lat_uy(oc), lg);
+        // Knuth's multiplicative hash, scaled to the positions
+        unsigned h = __umulhi(key * 2654435761u, (unsigned)RQ::HASH);
+        for (;; h = h + 1 < RQ::HASH ? h + 1 : 0) {
+          const unsigned old = atomicCAS(&rq.hash[h], RB_EMPTY, key);
           if (old == RB_EMPTY) {
-            const int slot = atomicAdd(&rq.nsolve, 1);
-            rq.hslot[h] = (unsigned short)slot;
-            rq.skey[slot] = key;
+            const unsigned slot = (unsigned)atomicAdd(&rq.nsolve, 1);
+            rq.spos[slot] = (unsigned short)h;
+            rq.hash[h] = key | slot << RQ::KEY_BITS;
             break;
           }
-          if (old == key) break;
+          if ((old & RB_KEY) == key) break;
         }
-        pos[j] = (unsigned short)h;
+        ent[j] = h << 16 | en;
       }
       __syncthreads();
       nsolve = rq.nsolve;
     }
-    // what to solve: the round's (sender, lattice) pairs, or the node
+    // what to solve: the round's (sender, lattice) pairs, or the node; wk and wc
+    // are the node whose multipliers start the solve and the solve's lattice
     NodeState s;
-    s.rho = -1.0;
+    NodeFields<P> nf;
     P lam[NM];
-    bool solve = false;
+    unsigned wk = (unsigned)k;
+    int wc = code;
+    bool solve = !rebuild && active;
     if (rebuild) {
       if (round + t < nsolve) {
-        const unsigned key = rq.skey[round + t];
-        const int oc = key >> 20;
-        const int Upx = lat_ux(oc), Upy = lat_uy(oc);
+        const unsigned key = rq.hash[rq.spos[round + t]] & RB_KEY;
+        const int at = (int)(key / 49u), w = (1 << lg) + 16;
+        wc = (int)(key % 49u);
         bool gh = false;
-        const int rx = resolve(x0 + (int)(key & 1023u) - 8, pr.nx, pr.bcx, &gh);
-        const int ry = resolve(y0 + (int)((key >> 10) & 1023u) - 8, pr.ny, pr.bcy, &gh);
-        const size_t ks = (size_t)ry * pr.nx + rx;
-        s.rho = (double)a.mom_in[ks];
-        s.ubx = (double)a.mom_in[ps + ks] - Upx;
-        s.uby = (double)a.mom_in[2 * ps + ks] - Upy;
-        s.T = (double)a.mom_in[3 * ps + ks];
-        if (pr.warm) load_warm<P>(a.lam_in, ps, ks, a.lat_in[ks], Upx, Upy, lam);
+        const int rx = resolve(x0 + at % w - 8, pr.nx, pr.bcx, &gh);
+        const int ry = resolve(y0 + at / w - 8, pr.ny, pr.bcy, &gh);
+        wk = (unsigned)ry * (unsigned)pr.nx + (unsigned)rx;
+        s.rho = (double)a.mom_in[wk];
+        s.ubx = (double)a.mom_in[ps + wk] - lat_ux(wc);
+        s.uby = (double)a.mom_in[2 * ps + wk] - lat_uy(wc);
+        s.T = (double)a.mom_in[3 * ps + wk];
         solve = true;
       }
     } else if (active) {
@@ -725,32 +819,32 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
       const bool by_nb = order_key(pr.overlap) > 0 && pr.rule == 1;
       if (by_nb) neighbour_codes(pr, a.nxt_in, x, y, nb);
       s = node_moments<P, B>(pr, cl, code, by_nb ? nb : nullptr);
-      if (pr.warm)
-        load_warm<P>(a.lam_in, ps, k, a.lat_in[k], lat_ux(code), lat_uy(code), lam);
-      solve = true;
+      nf = node_publish<P>(code, s, k, ps, a.mom_out, a.lat_out, a.nxt_out);
     }
     int st = NEWTON_UNREALIZABLE;
     bool fixed = false;
     if (solve) {
-      nc.calls += 1;
-      if (s.rho > 0.0)
-        st = node_equilibrium<P, B>(pr, cl, s.ubx, s.uby, s.T, pr.warm, lam, &nc.solve, &fixed);
+      nc.n += N_CALLS;
+      st = node_equilibrium<P, B>(
+          pr, cl, s, pr.warm,
+          [&](P* l) { load_warm<P>(a.lam_in, ps, wk, a.lat_in[wk], lat_ux(wc), lat_uy(wc), l); },
+          lam, &nc, a.ctr, &fixed);
     }
     if (!rebuild) {
-      if (active)
-        node_store<P, B>(pr, cl, code, s, st, fixed, pr.warm, lam, k, ps, a.pop_out, a.mom_out,
-                         a.lat_out, a.nxt_out, a.lam_out, &nc.fail);
+      if (active && !node_store<P, B>(pr, cl, nf, st, fixed, pr.warm, lam, k, ps, a.pop_out,
+                                      a.lam_out))
+        nc.n |= N_FAIL;
       break;
     }
     rq.state[t] = (unsigned char)((st == NEWTON_OK ? 0 : 1) | (fixed ? 2 : 0));
     __syncthreads();
 #pragma unroll 1
     for (int j = 0; j < RQ::PER; ++j) {
-      const int e = base + j * B + t;
-      if (e >= nq) break;
-      const int j0 = (int)rq.hslot[j == 0 ? pos[0] : j == 1 ? pos[1] : pos[2]] - round;
+      if (base + j * B + t >= nq) break;
+      const unsigned en = j == 0 ? ent[0] : j == 1 ? ent[1] : ent[RQ::PER - 1];
+      const int j0 = (int)(rq.hash[en >> 16] >> RQ::KEY_BITS) - round;
       if (j0 < 0 || j0 >= B) continue;  // solved in another round
-      const int owner = rq.entry[e] >> 5, i = rq.entry[e] & 31;
+      const int owner = (en >> 5) & 255, i = en & 31;
       const int ox = x0 + (owner & mask), oy = y0 + (owner >> lg);
       const int oc = a.nxt_in[(size_t)oy * pr.nx + ox];
       const int Upx = lat_ux(oc), Upy = lat_uy(oc);
@@ -761,8 +855,7 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
       double fd, gd;
       rebuild_value<P>(pr, a.mom_in, ps, cx, cy, Upx, Upy, ox - cx - Upx, oy - cy - Upy, eq, ok,
                        &fd, &gd);
-      nc.rec += 1;
-      nc.rec_fail += ok ? 0 : 1;
+      nc.n += ok ? N_REC : N_REC + N_REC_FAIL;
       pop0[i * B + owner] = (P)fd;
       pop0[(Q + i) * B + owner] = (P)gd;
     }
