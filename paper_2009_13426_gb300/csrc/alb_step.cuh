@@ -160,16 +160,28 @@ __device__ __forceinline__ int node_equilibrium(const Params& pr, const Columns<
                      reinterpret_cast<uint64_t*>(cl.eq), B, lam, &nc->fix);
     *fixed = st == NEWTON_OK;
     if (st != NEWTON_OK) {
+      // A refinement that did not take the state leaves multipliers that the FP32
+      // phase has converged: the other solve starts there (states near the edge
+      // of what the lattice carries take up to 30 FP32 steps, and have the
+      // exponents the fixed-point range ends at).
       SolveIO io;
       io.ubx = ubx;
       io.uby = uby;
       io.T = T;
-      io.warm = warm;
-      if (warm) load(io.lam);
+      const bool converged = st == NEWTON_MAXIT;
+      io.warm = warm || converged;
+      if (converged)
+#pragma unroll
+        for (int k = 0; k < NM; ++k) io.lam[k] = lam[k];
+      else if (warm)
+        load(io.lam);
       st = solve_other<B>(pr, cl.exptab, cl.fixtab, cl.eq, &io, ctr);
       *fixed = io.fixed;
+      if (st == NEWTON_OK || !warm)
 #pragma unroll
-      for (int k = 0; k < NM; ++k) lam[k] = io.lam[k];
+        for (int k = 0; k < NM; ++k) lam[k] = io.lam[k];
+      else
+        load(lam);
     }
     return st;
   } else {
