@@ -278,6 +278,41 @@ __device__ __forceinline__ void grad_phi(const Params& pr, double rho, double T,
   *phi_g = mul_rn(mul_rn(2.0, qc), irc);
 }
 
+// Grad's factors as polynomials of the lattice velocity xi = c_i - U: with cbar = xi
+// - ubar, phi_f has the eight monomials P_k (a), phi_g is linear (g). All 21
+// factors then take some 100 operations instead of 30 each.
+__device__ __forceinline__ void grad_poly(const Params& pr, double rho, double T, double ubx,
+                                          double uby, const double du[2][2], const double dT[2],
+                                          double a[NM], double g[3]) {
+  const double iT = 1.0 / T, irho = 1.0 / rho;
+  const double mu = rho * pr.nu, kappa = rho * pr.cp * pr.kappa_nu;
+  const double div = du[0][0] + du[1][1];
+  const double irc = irho * pr.icp, iT2 = iT * iT;
+  const double s0 = 0.5 * iT2 * irho;
+  // stress: A cx^2 + B cx cy + C cy^2
+  const double A = -s0 * mu * (2.0 * du[0][0] - div), C = -s0 * mu * (2.0 * du[1][1] - div);
+  const double Bq = -2.0 * s0 * mu * (du[0][1] + du[1][0]);
+  // heat flux: (Qx cx + Qy cy) (h |cbar|^2 - cp), with cbar expanded as
+  // (Qx x + Qy y - L0) (h r^2 - n1 x - n2 y + n0)
+  const double k1 = -iT2 * irc * kappa, h = 0.5 * iT;
+  const double Qx = k1 * dT[0], Qy = k1 * dT[1];
+  const double L0 = Qx * ubx + Qy * uby;
+  const double n1 = 2.0 * h * ubx, n2 = 2.0 * h * uby;
+  const double n0 = h * (ubx * ubx + uby * uby) - pr.cp;
+  a[0] = A * ubx * ubx + Bq * ubx * uby + C * uby * uby - L0 * n0;
+  a[1] = -2.0 * A * ubx - Bq * uby + Qx * n0 + L0 * n1;
+  a[2] = -2.0 * C * uby - Bq * ubx + Qy * n0 + L0 * n2;
+  a[3] = A - Qx * n1 - L0 * h;
+  a[4] = Bq - Qx * n2 - Qy * n1;
+  a[5] = C - Qy * n2 - L0 * h;
+  a[6] = Qx * h;
+  a[7] = Qy * h;
+  const double k2 = -2.0 * irc * kappa;
+  g[1] = k2 * dT[0];
+  g[2] = k2 * dT[1];
+  g[0] = -(g[1] * ubx + g[2] * uby);
+}
+
 // Resolve a coordinate along one axis: periodic wrap or zero-gradient clamp.
 __device__ __forceinline__ int resolve(int x, int n, int bc, bool* ghost) {
   if (bc == 0) {

@@ -55,6 +55,50 @@ __device__ __forceinline__ void init_prim(const double* rho, const double* rhoux
   *T = (rhoE[k] - 0.5 * (*r) * ((*ux) * (*ux) + (*uy) * (*uy))) / ((*r) * cv);
 }
 
+// The same at a neighbour, for the central differences of u and T: one reciprocal
+// instead of three divisions (the node's own velocity, which chooses its lattice,
+// keeps the divisions).
+__device__ __forceinline__ void init_near(const double* rho, const double* rhoux,
+                                          const double* rhouy, const double* rhoE, double icv,
+                                          size_t k, double* ux, double* uy, double* T) {
+  const double ir = 1.0 / rho[k];
+  *ux = rhoux[k] * ir;
+  *uy = rhouy[k] * ir;
+  *T = (rhoE[k] * ir - 0.5 * ((*ux) * (*ux) + (*uy) * (*uy))) * icv;
+}
+
+// Visitor that writes the Grad-regularised populations of a node to its column:
+// s = 1 + phi_f of every velocity (grad_poly).
+template <typename P>
+struct GradFill {
+  P* pop;
+  const double* eq;
+  bool fixed;
+  double r, gfac, g0, gx, gy;
+  __device__ __forceinline__ GradFill(P* p, const double* e, bool fx, double r_, double gf,
+                                      const double g[3])
+      : pop(p), eq(e), fixed(fx), r(r_), gfac(gf), g0(1.0 + g[0]), gx(g[1]), gy(g[2]) {}
+  template <int I>
+  __device__ __forceinline__ void put(double s) {
+    const double feq = r * eq_f64<P>(eq[I * BLOCK], fixed);
+    pop[I * BLOCK] = to_p<P>(feq * s);
+    pop[(Q + I) * BLOCK] = to_p<P>(gfac * feq * madd(madd(g0, gx, XI_X(I)), gy, XI_Y(I)));
+  }
+  __device__ __forceinline__ void rest(double s) { put<0>(s); }
+  template <int A, int AX, int IP, int IM>
+  __device__ __forceinline__ void pair(double sp, double sm) {
+    put<IP>(sp);
+    put<IM>(sm);
+  }
+  template <int A, int IPP, int IMP, int IMM, int IPM>
+  __device__ __forceinline__ void quad(double spp, double smp, double smm, double spm) {
+    put<IPP>(spp);
+    put<IMP>(smp);
+    put<IMM>(smm);
+    put<IPM>(spm);
+  }
+};
+
 // Grad-regularised initial condition (Sec. IV.A.1): h = h^eq (1 + phi_h) in the
 // lattice chosen from the initial velocity, then the first collision.
 template <typename P>
@@ -73,16 +117,17 @@ __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1)
     bool gh = false;
     const int xp = resolve(x + 1, pr.nx, pr.bcx, &gh), xm = resolve(x - 1, pr.nx, pr.bcx, &gh);
     const int yp = resolve(y + 1, pr.ny, pr.bcy, &gh), ym = resolve(y - 1, pr.ny, pr.bcy, &gh);
-    double r, ux, uy, T, r1, ux1, uy1, T1, r2, ux2, uy2, T2;
+    double r, ux, uy, T, ux1, uy1, T1, ux2, uy2, T2;
     init_prim(a.rho, a.rhoux, a.rhouy, a.rhoE, pr.cv, k, &r, &ux, &uy, &T);
     double du[2][2], dT[2];
-    init_prim(a.rho, a.rhoux, a.rhouy, a.rhoE, pr.cv, y * nx + xp, &r1, &ux1, &uy1, &T1);
-    init_prim(a.rho, a.rhoux, a.rhouy, a.rhoE, pr.cv, y * nx + xm, &r2, &ux2, &uy2, &T2);
+    const double icv = pr.gamma - 1.0;
+    init_near(a.rho, a.rhoux, a.rhouy, a.rhoE, icv, y * nx + xp, &ux1, &uy1, &T1);
+    init_near(a.rho, a.rhoux, a.rhouy, a.rhoE, icv, y * nx + xm, &ux2, &uy2, &T2);
     du[0][0] = 0.5 * (ux1 - ux2);
     du[0][1] = 0.5 * (uy1 - uy2);
     dT[0] = 0.5 * (T1 - T2);
-    init_prim(a.rho, a.rhoux, a.rhouy, a.rhoE, pr.cv, yp * nx + x, &r1, &ux1, &uy1, &T1);
-    init_prim(a.rho, a.rhoux, a.rhouy, a.rhoE, pr.cv, ym * nx + x, &r2, &ux2, &uy2, &T2);
+    init_near(a.rho, a.rhoux, a.rhouy, a.rhoE, icv, yp * nx + x, &ux1, &uy1, &T1);
+    init_near(a.rho, a.rhoux, a.rhouy, a.rhoE, icv, ym * nx + x, &ux2, &uy2, &T2);
     du[1][0] = 0.5 * (ux1 - ux2);
     du[1][1] = 0.5 * (uy1 - uy2);
     dT[1] = 0.5 * (T1 - T2);
@@ -98,21 +143,11 @@ __global__ void __launch_bounds__(BLOCK, (std::is_same<P, float>::value ? 4 : 1)
                        : NEWTON_UNREALIZABLE;
     if (!realizable) n_bad += 1;
     if (ns != NEWTON_OK && realizable) n_fail += 1;
-    const double gfac = (2.0 * pr.cv - 2.0) * T;
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-      const double cbx = (double)(XI_X(i) + U0x) - ux;
-      const double cby = (double)(XI_Y(i) + U0y) - uy;
-      double phf = 0.0, phg = 0.0, phq = 0.0;
-      double feq = 0.0;
-      if (ns == NEWTON_OK) {
-        grad_phi(pr, r, T, cbx, cby, du, dT, &phf, &phg, &phq);
-        feq = r * eq_f64<P>(cl.eq[i * BLOCK], fixed);
-      }
-      cl.pop[i * BLOCK] = (P)(feq * (1.0 + phf));
-      cl.pop[(Q + i) * BLOCK] = (P)(gfac * feq * (1.0 + phg));
-    }
     if (ns == NEWTON_OK) {
+      double ca[NM], cg[3];
+      grad_poly(pr, r, T, ux - U0x, uy - U0y, du, dT, ca, cg);
+      GradFill<P> fill(cl.pop, cl.eq, fixed, r, (2.0 * pr.cv - 2.0) * T, cg);
+      visit_groups<double>(ca, fill);
       // the first collision starts from the multipliers just found if the
       // flow starts its solves from previous multipliers
       // with the neighbourhood rule, the neighbours' initial lattices (Eq.
