@@ -177,11 +177,12 @@ cudaError_t GroupPlan::flip(cudaStream_t s) const { return launch_flip(d_cur_, n
     if (e_ != cudaSuccess) return cuda_error(e_, what);     \
   } while (0)
 
-// Default launch shape of a precision: the single-flow kernel's block in the FP32
-// form (variant 2, 256 x 2), variant 0 in FP64 plain; tiles 32 nodes wide.
+// Default launch shape of a precision: 256 threads without spills in the FP32 form
+// (variant 4; see launch_step for the shapes by size), variant 0 in FP64 plain;
+// tiles 32 nodes wide.
 Tuning default_tuning(int precision) {
   Tuning t;
-  if (precision == ALB_FP32_FORM) t.variant = 2;
+  if (precision == ALB_FP32_FORM) t.variant = 4;
   const int block = batch_variant(precision, t.variant).block;
   for (int c = 0; c < 3; ++c) t.tile_w[c] = std::min(t.tile_w[c], block);
   return t;
@@ -231,7 +232,7 @@ static int try_tuning(cudaStream_t stream, GroupPlan* p, const Tuning& t, int on
 
 
 // Coordinate search of one precision's launch shape: the kernel variant
-// (tiles as wide as the block), then the tile width of each size class
+// (tiles 32 nodes wide), then the tile width of each size class
 // present (timing only that class's items), then static against dynamic work
 // distribution. The plan ends with the best shape found (the default one
 // after an error) and a full item table.
@@ -526,8 +527,8 @@ int alb_batch_set_tuning(alb_batch* b, int precision, const alb_batch_tuning* t)
   return ALB_OK;
 }
 
-// Coordinate search, per precision: the kernel variant (tiles as wide as
-// possible), then the tile width of each size class present (timing only
+// Coordinate search, per precision: the kernel variant (tiles 32 nodes
+// wide), then the tile width of each size class present (timing only
 // that class's items), then static against dynamic work distribution.
 int alb_batch_tune(alb_batch* b, int trials) {
   if (!b) return set_error(ALB_EINVAL, "alb_batch_tune: null batch");

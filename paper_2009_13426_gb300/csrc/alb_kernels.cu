@@ -344,25 +344,33 @@ static cudaError_t launch_step_shape(const FlowDev& f, cudaStream_t s) {
 // nodes of 256, where the longer rounds of rebuild solves save more than the
 // second block hides (64^2 vortex 0.39 against 0.42 ms, 201^2 Riemann 0.45 / 0.56,
 // 512^2 shear 1.44 / 1.46, but 700^2 2.53 / 2.46 and 1400^2 vortex 7.73 / 7.39).
-constexpr size_t FP64_SMALL = 512 * 512;
+//
+// FP32 form, ms a step with 256 threads and 255 registers (one block per SM),
+// 384 and 168, and two blocks of 256 and 128, which spill but keep 16 warps:
+//   64^2 vortex 0.103 / 0.149 / 0.127    201^2 Riemann 0.105 / 0.121 / 0.131
+//   512^2 shear 0.260 / 0.277 / 0.283    700^2 shear 0.376 / 0.368 / 0.419
+//   1021 x 733 shear 0.567 / 0.545 / 0.580   1400^2 vortex 1.01 / 0.97 / 0.90
+//   4096^2 shear 9.94 / 9.68 / 10.0
+// Few tiles want the shortest chain through one block, many the most warps.
+// Blocks smaller than 256 lose threads for an interface tile's rebuild solves
+// (201^2: 0.161 with 128, 0.207 with 64 where 256 took 0.151). Grids of fewer
+// than 8 rows do not fill the 32 x 8 tile: 128 threads (2048 x 4 tube 0.048 ms).
+constexpr size_t FP64_SMALL = 512 * 512, FP32_SMALL = 512 * 512, FP32_MEDIUM = 1024 * 1024;
 
-// Block size of the FP32 form: 256 threads, two blocks per SM. Smaller blocks
-// would fill more SMs on a small grid, but an interface tile has then fewer
-// threads for its rebuild solves, which are the longest chain of such a step
-// (64^2 vortex 0.146 ms against 0.153 with 128 and 0.180 with 64 threads,
-// 201^2 Riemann 0.151 / 0.161 / 0.207, 512^2 shear 0.31 / 0.42 / 0.58; blocks of
-// 512 measured 0.174, 0.166 and 0.345). Grids of fewer than 8 rows do not fill
-// the 32 x 8 tile: 128 threads (2048 x 4 tube 0.059 ms against 0.087).
 cudaError_t launch_step(FlowDev& f, cudaStream_t s) {
   if (f.q == 49) return launch_step_q49(f, s);
   cudaError_t e;
   if (f.precision == 0)
     e = f.n <= FP64_SMALL && f.prm.ny >= 8 ? launch_step_shape<double, 256, 1>(f, s)
                                            : launch_step_shape<double, 128, 1>(f, s);
-  else if (f.prm.ny >= 8)
-    e = launch_step_shape<float, 256, 2>(f, s);
+  else if (f.prm.ny < 8)
+    e = launch_step_shape<float, 128, 2>(f, s);
+  else if (f.n <= FP32_SMALL)
+    e = launch_step_shape<float, 256, 1>(f, s);
+  else if (f.n <= FP32_MEDIUM)
+    e = launch_step_shape<float, 384, 1>(f, s);
   else
-    e = launch_step_shape<float, 128, 4>(f, s);
+    e = launch_step_shape<float, 256, 2>(f, s);
   if (e == cudaSuccess) f.cur ^= 1;
   return e;
 }

@@ -623,8 +623,8 @@ struct RebuildQueue {
   __device__ __forceinline__ unsigned entry(int e) const {
     int o = 0;
 #pragma unroll
-    for (int d = B / 2; d > 0; d >>= 1)
-      if (start[o + d] <= e) o += d;
+    for (int d = B > 256 ? 256 : B > 128 ? 128 : 64; d > 0; d >>= 1)
+      if (o + d < B && start[o + d] <= e) o += d;
     unsigned m = miss[o];
     for (int j = e - start[o]; j > 0; --j) m &= m - 1;
     return (unsigned)o << 5 | (unsigned)(__ffs(m) - 1);
@@ -763,7 +763,7 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
   // run B at a time in the columns of threads 0, 1, ...; every entry then takes
   // its value from the column of its solve (which entry comes first into the
   // table, and which thread solves it, changes no value).
-  static_assert(B % 32 == 0 && B <= 256, "whole warps; 13 bits for an entry");
+  static_assert(B % 32 == 0 && B <= 512, "whole warps; 14 bits for an entry");
   using RQ = RebuildQueue<P, B>;
   P* const pop0 = cl.pop - t;  // column 0 of the block
   int base = 0, round = 0, nsolve = 0;  // chunk, its solves done, its solves
@@ -856,7 +856,7 @@ __device__ __forceinline__ void tile_step(const StepArgs<P>& a, int x0, int y0, 
       const unsigned en = j == 0 ? ent[0] : j == 1 ? ent[1] : ent[RQ::PER - 1];
       const int j0 = (int)(rq.hash[en >> 16] >> RQ::KEY_BITS) - round;
       if (j0 < 0 || j0 >= B) continue;  // solved in another round
-      const int owner = (en >> 5) & 255, i = en & 31;
+      const int owner = (en >> 5) & 511, i = en & 31;
       const int ox = x0 + (owner & mask), oy = y0 + (owner >> lg);
       const int oc = a.nxt_in[(size_t)oy * pr.nx + ox];
       const int Upx = lat_ux(oc), Upy = lat_uy(oc);
