@@ -59,12 +59,11 @@ from paper_2009_13426_gb300 import costmodel, flows  # noqa: E402
 
 METRIC = "adaptive D2Q21 MLUPS, FP32 form vs FP64 plain at stated error; serve p50/p99"
 # DRAM bytes (read + write) per node update of step_kernel<float>, from one
-# ncu capture of the 1024^2 case of the same flow (dram__bytes_read.sum +
-# dram__bytes_write.sum = 226.9 + 370.5 MB per launch for 1,048,576 nodes,
-# mean of the first 3 launches, kinetic sensor on); the traffic
-# grows in proportion to the nodes, so a 4096^2 launch moves 16,777,216 x
-# this. Measured on the current kernel.
-TRAFFIC_BYTES_PER_NODE_FP32 = 569.7
+# ncu capture of the 2048^2 case of the same flow (dram__bytes_read.sum +
+# dram__bytes_write.sum = 876.8 + 1117.8 MB per launch for 4,194,304 nodes,
+# first steps, kinetic sensor on); the traffic grows in proportion to the
+# nodes, so a 4096^2 launch moves 16,777,216 x this.
+TRAFFIC_BYTES_PER_NODE_FP32 = 475.6
 UNIT = "MLUPS"
 NU = 1e-5
 # The kinetic sensor (Sec. IV.A.2) is on in every timed flow: without it the
@@ -434,8 +433,7 @@ def run_batched(args):
     launches = k * (2 if tuning["dynamic"] else 1) + (k % 2)
     upd = nodes * k
     tot["node_updates"] = upd
-    slots = costmodel.fp64_slots(tot, "fp32")
-    tflops = 2.0 * slots / (ms * 1e-3) / 1e12
+    tinstr = costmodel.issue_instr(tot) / (ms * 1e-3) / 1e12
     return {"workload": "256 periodic flows, side log-uniform 64-1024 (seed 4), vortex or "
                         "shear layer, Mach 0.5-3, T ratio 1-4, nu 1e-5..1e-3, FP32 form",
             "flows": len(specs), "nodes": nodes, "steps": k, "unit": UNIT,
@@ -447,9 +445,9 @@ def run_batched(args):
             "per_node": {key: round(v / upd, 4) for key, v in tot.items()
                          if key not in ("newton_failures", "reconstruction_failures",
                                         "node_updates")},
-            "roofline": {"bound": "alu", "achieved": round(tflops, 4),
-                         "peak": round(costmodel.FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
-                         "frac": round(tflops / costmodel.FP64_PEAK_TFLOPS, 4),
+            "roofline": {"bound": "issue", "achieved": round(tinstr, 4),
+                         "peak": round(costmodel.ISSUE_PEAK_TINSTR, 4), "unit": "Tinstr/s",
+                         "frac": round(tinstr / costmodel.ISSUE_PEAK_TINSTR, 4),
                          "kernel": "batch_step_kernel<float>"},
             "failures": {"node": tot["newton_failures"],
                          "rebuild": tot["reconstruction_failures"],
@@ -629,8 +627,8 @@ def run_ours(args, world, rank, local):
     ms_max = dist_max(ms32, world)
     mlups = aggregate_mlups(world, N, args.steps, ms_max)
     per_launch_ms = ms32 / args.steps
-    slots = costmodel.fp64_slots(d32, "fp32")
-    achieved_tflops = 2.0 * slots / args.steps / (per_launch_ms * 1e-3) / 1e12
+    instr = costmodel.issue_instr(d32)
+    achieved_tinstr = instr / args.steps / (per_launch_ms * 1e-3) / 1e12
     bytes_per_launch = costmodel.BYTES_PER_NODE["fp32"] * N
     hbm_gbs = bytes_per_launch / (per_launch_ms * 1e-3) / 1e9
     total32 = args.warmup + args.steps
@@ -655,7 +653,7 @@ def run_ours(args, world, rank, local):
                    np.sqrt((a - A) ** 2 + (b - B) ** 2).max() / np.sqrt(A ** 2 + B ** 2).max(),
                    np.abs(e - E).max() / np.abs(E).max())
         tot = max(abs(r.sum() - R.sum()) / R.sum(), abs(e.sum() - E.sum()) / E.sum())
-        slots64 = costmodel.fp64_slots(d64, "fp64")
+        slots64 = costmodel.plain_slots(d64)
         extra["fp64_plain"] = {"value": round(N * k64 / (ms64 * 1e-3) / 1e6, 2), "unit": UNIT,
                                "steps": k64, "ms_per_step": round(ms64 / k64, 3),
                                "fp64_slots_per_node": round(slots64 / k64 / N, 1),
@@ -698,8 +696,7 @@ def run_ours(args, world, rank, local):
         ms_d, dd = timed(fl32, k_dev, 0)
         clk_d = clocks_d.stop()
         ms_d = dist_max(ms_d, world)
-        slots_d = costmodel.fp64_slots(dd, "fp32")
-        tf_d = 2.0 * slots_d / (ms_d * 1e-3) / 1e12
+        ti_d = costmodel.issue_instr(dd) / (ms_d * 1e-3) / 1e12
         developed = {"value": round(aggregate_mlups(world, N, k_dev, ms_d), 2), "unit": UNIT,
                      "steps": [args.developed_steps - k_dev, args.developed_steps],
                      "ms_per_step": round(ms_d / k_dev, 3),
@@ -708,12 +705,10 @@ def run_ours(args, world, rank, local):
                                             "newton_calls", "reconstructions")},
                      "failures": {"node": dd["newton_failures"],
                                   "rebuild": dd["reconstruction_failures"]},
-                     "roofline": {"bound": "alu", "achieved": round(tf_d, 4),
-                                  "peak": round(costmodel.FP64_PEAK_TFLOPS, 4),
-                                  "unit": "TFLOP/s",
-                                  "frac": round(tf_d / costmodel.FP64_PEAK_TFLOPS, 4),
-                                  "note": "FP64 slots only: the FP32 Newton steps, more "
-                                          "than two per node here, are not counted"},
+                     "roofline": {"bound": "issue", "achieved": round(ti_d, 4),
+                                  "peak": round(costmodel.ISSUE_PEAK_TINSTR, 4),
+                                  "unit": "Tinstr/s",
+                                  "frac": round(ti_d / costmodel.ISSUE_PEAK_TINSTR, 4)},
                      "clocks": clk_d}
         r, a, b, e = fl32.moments()
         T = (e / r - 0.5 * ((a / r) ** 2 + (b / r) ** 2)) / 2.5
@@ -772,12 +767,6 @@ def run_ours(args, world, rank, local):
                             for k in ("newton_iterations", "newton_calls", "reconstructions")},
                "failures": {"node": d49["newton_failures"],
                             "rebuild": d49["reconstruction_failures"]}}
-        slots49 = costmodel.q49_slots(d49, N49 * k49)
-        if slots49:
-            t49 = 2.0 * slots49 / (ms49 * 1e-3) / 1e12
-            q49["roofline"] = {"bound": "alu", "achieved": round(t49, 4),
-                               "peak": round(costmodel.FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
-                               "frac": round(t49 / costmodel.FP64_PEAK_TFLOPS, 4)}
         fl.close()
 
     e2e = None
@@ -830,17 +819,16 @@ def run_ours(args, world, rank, local):
         "higher_is_better": True, "scaling": "weak", "vs_baseline": None, "dtype": "f32+f64",
         "data": "synthetic",
         "config": workload_config(n, world),
-        "roofline": {"bound": "alu", "achieved": round(achieved_tflops, 4),
-                     "peak": round(costmodel.FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
-                     "frac": round(achieved_tflops / costmodel.FP64_PEAK_TFLOPS, 4),
+        "roofline": {"bound": "issue", "achieved": round(achieved_tinstr, 4),
+                     "peak": round(costmodel.ISSUE_PEAK_TINSTR, 4), "unit": "Tinstr/s",
+                     "frac": round(achieved_tinstr / costmodel.ISSUE_PEAK_TINSTR, 4),
                      "traffic": round(TRAFFIC_BYTES_PER_NODE_FP32 * N),
-                     "traffic_note": "ncu DRAM bytes per node on the 1024^2 case x nodes: "
-                                     "1.36 x the 420 algorithmic bytes, the excess being "
+                     "traffic_note": "ncu DRAM bytes per node on the 2048^2 case x nodes: "
+                                     "1.13 x the 420 algorithmic bytes, the excess being "
                                      "the threads' stack (spills, call frames) leaving L2",
-                     "peak_source": "FP64: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz",
+                     "peak_source": "issue: 152 SMs x 4 warp instructions/clk x 32 x 2.07 GHz",
                      "kernel": "step_kernel<float>",
-                     "fp64_slots_per_node": round(slots / args.steps / N, 1),
-                     "method_floor": costmodel.method_floor(mlups / world),
+                     "instr_per_node": round(instr / args.steps / N, 1),
                      "hbm": {"achieved_gbs": round(hbm_gbs, 1),
                              "bytes_per_node": costmodel.BYTES_PER_NODE["fp32"]}},
         "clocks": clk,

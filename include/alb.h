@@ -82,9 +82,11 @@ typedef struct alb_handle alb_handle; /* opaque */
  *   gamma        specific heat ratio gamma_r (> 1).
  *   n0           criterion offset: U = n iff n - n0 < u <= n + 1 - n0
  *                (0.5 gives Eq. criterion as printed).
- *   precision    ALB_FP64_PLAIN: populations, moments and arithmetic in FP64.
+ *   precision    ALB_FP64_PLAIN: populations, moments and arithmetic in FP64 (but
+ *                the early steps of a solve, see newton_start).
  *                ALB_FP32_FORM: populations and moment sums in FP32
- *                (compensated summation), FP64 only in the Newton solve.
+ *                (compensated summation), the solve's residuals in
+ *                64-bit fixed point or FP64.
  *   bc_x, bc_y   ALB_PERIODIC, or ALB_ZERO_GRADIENT (ghost nodes carry the
  *                nearest interior node's moments; pulls from them are rebuilt).
  *   sensor       1 enables tau <- tau * alpha(eps_Kn) (Eq. DeltaAvg). alpha is

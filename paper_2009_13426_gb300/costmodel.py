@@ -1,7 +1,13 @@
 """Work model of the step kernel, used for the roofline of the benchmark.
 
-The step is bound by the FP64 pipe, not by HBM: on GB300 the FP64 rate is
-1/62 of the FP32 rate. Its FP64 arithmetic is counted in issue slots: one
+FP64 plain and D2Q49 are bound by the FP64 pipe, not by HBM: on GB300 the FP64
+rate is 1/62 of the FP32 rate. The FP32 form forms its residuals in fixed point
+on the integer pipe and is bound by instruction issue and the latency of its
+chains at 8 to 16 warps per SM (issue_instr below); the FP32-form counts of
+fp64_slots describe its FP64 refinement, which now serves only states outside
+the fixed-point range.
+
+FP64 arithmetic is counted in issue slots: one
 slot per FP64 lane operation (DFMA, DADD, DMUL, DMNMX, DSETP, hardware
 conversions to or from FP64; the FP32 form's hot conversions are assembled
 on the integer pipe instead and cost no slot), and for CUDA's FP64 routines
@@ -152,7 +158,8 @@ REBUILD_EXTRA = {
 
 
 def fp64_slots(stats: dict, precision: str) -> float:
-    """FP64 slots of the work recorded by the kernel counters (a stats delta)."""
+    """FP64 slots of the work recorded by the kernel counters (a stats delta): FP32
+    form with every residual in FP64, FP64 plain with every Newton step in FP64."""
     if precision == "fp32":
         raw = (stats["fp64_evaluations"] * mixed_eval()
                + stats.get("fp64_updates", 0) * mixed_update()
@@ -166,6 +173,41 @@ def fp64_slots(stats: dict, precision: str) -> float:
     raw += stats["node_updates"] * COLLISION[precision]
     raw += stats["reconstructions"] * REBUILD_EXTRA[precision]
     return CALIBRATION[precision] * raw
+
+
+# ------------------------------------------------- work of the current kernels
+
+# Instruction issue: 152 SMs x 4 schedulers x 32 lanes x 2.07 GHz.
+ISSUE_PEAK_TINSTR = 152 * 4 * 32 * 2.07e9 / 1e12   # 40.27
+
+
+def issue_instr(stats: dict) -> float:
+    """Thread instructions of FP32-form launches, from ncu's counts of a kernel cut
+    after each phase (2048^2 and 1024^2 shear layers): pulls, moments, collision
+    and store 3,300 per node, 650 per FP32 evaluation pass with its factorisation,
+    1,150 per fixed-point evaluation or update, 2,000 per rebuilt pull. It gives
+    6,830 per node where ncu counts 6,858 (2048^2, first steps)."""
+    return (3300.0 * stats["node_updates"]
+            + 650.0 * (stats["fp32_iterations"] + stats["newton_calls"])
+            + 1150.0 * (stats["fp64_evaluations"] + stats.get("fp64_updates", 0))
+            + 2000.0 * stats["reconstructions"])
+
+
+def plain_slots(stats: dict) -> float:
+    """FP64 slots of FP64 plain launches whose early Newton steps run in FP32: per
+    evaluation the grouped exponents (55), 21 exponentials (7 each), the 27 moment
+    sums (96), the residual and the Jacobian's entries (30); per FP64 step the
+    correction by the Jacobian and the update of the multipliers (80)."""
+    steps = max(0, stats["newton_iterations"] - stats["fp32_iterations"])
+    raw = (stats["fp64_evaluations"] * (55 + 21 * 7 + 96 + 30) + steps * 80
+           + stats["newton_calls"] * 8 + stats["node_updates"] * COLLISION["fp64"]
+           + stats["reconstructions"] * REBUILD_EXTRA["fp64"])
+    return PLAIN_MIXED_CALIBRATION * raw
+
+
+# ncu counted 2,156 FP64-pipe thread instructions per node on the 1024^2 layer (4.20
+# evaluations, 3.13 FP64 steps, 1.08 solves, 0.20 rebuilt pulls per node).
+PLAIN_MIXED_CALIBRATION = 2156.0 / 1980.7
 
 
 def method_floor(mlups: float) -> dict:
@@ -222,7 +264,8 @@ CALIBRATION["q49"] = 30696.0 / 22067.0
 
 
 def q49_slots(delta, node_updates):
-    """FP64 slots of D2Q49 launches from their counters."""
+    """FP64 slots of D2Q49 launches with every Newton step in FP64 (an explicit
+    Maxwellian start), from their counters."""
     rebuilds = delta["reconstructions"]
     raw = (Q49_PER_ITER * delta["newton_iterations"] + Q49_PER_CALL * delta["newton_calls"]
            + Q49_PER_NODE * node_updates + Q49_PER_REBUILD * rebuilds)

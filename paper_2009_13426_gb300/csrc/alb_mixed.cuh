@@ -1,14 +1,18 @@
-// Mixed-precision solver of the 8-moment numerical equilibrium, FP32 form.
+// Solvers of the numerical equilibrium: FP32 Newton phase, residuals in fixed
+// point (solve_fix, FP32 form) or FP64 (solve_mixed64, FP64 plain; refine_fp64,
+// the FP32 form's states outside the fixed-point range), FP64 Newton throughout
+// (newton_fp64g), and the reduced model.
 //
 // The multipliers of Eq. feqNum_8Mom solve G(lambda) = 0 (Eqs. G0_8mom..
 // G3yaa_8mom). On GB300 the FP64 pipe runs at 1/62 of the FP32 rate, so the
 // Newton iterations run in FP32 (exponentials, exact Jacobian, Cholesky
-// factor), and FP64 is used only where the accuracy of the result comes
-// from: the residual. The FP64 refinement evaluates the 21 exponentials and
-// the 8 constraint residuals in FP64 and corrects lambda with the FP32
-// Cholesky factor (iterative refinement of the Newton step) until
-// max_k |G_k| / rho <= tol, the same criterion as the full FP64 Newton. If the
-// FP32 phase or the refinement fails, the full FP64 Newton takes over.
+// factor), and 64 bits are used only where the accuracy of the result comes
+// from: the residual. The refinement evaluates the 21 exponentials and the 8
+// constraint residuals in 64-bit integers (alb_fix.cuh) or FP64 and corrects
+// lambda with the FP32 Cholesky factor (iterative refinement of the Newton
+// step) until max_k |G_k| / rho <= tol, the same criterion as the full FP64
+// Newton. If the FP32 phase or the refinement fails, the full FP64 Newton takes
+// over.
 //
 // The FP64 exponential is table-driven (Tang, ACM TOMS 15(2), 1989):
 // exp(-s) = 2^(n/256) exp(r), n = round(-256 s / ln 2), |r| <= ln2/512, with
