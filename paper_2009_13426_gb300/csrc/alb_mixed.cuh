@@ -224,6 +224,14 @@ __device__ __forceinline__ Exp2 fma(Exp2 a, Exp2 b, Exp2 c) {
 }  // namespace dual
 using dual::Exp2;
 
+// Maximum that is NaN if either argument is (fmaxf drops a NaN, so that residuals
+// that are all NaN would have the maximum 0 and pass for converged).
+__device__ __forceinline__ float max_nan(float a, float b) {
+  float r;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+  return r;
+}
+
 // Packed lower triangle of the 8x8 Jacobian: entry (a, b), b <= a.
 __host__ __device__ constexpr int tri(int a, int b) { return a * (a + 1) / 2 + b; }
 
@@ -805,7 +813,7 @@ __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int ma
 #pragma unroll
     for (int k = 0; k < NM; ++k) {
       G[k] -= m[k];
-      gmax = fmaxf(gmax, fabsf(G[k]));
+      gmax = max_nan(gmax, fabsf(G[k]));
     }
     *gres = gmax;
     if (!FACTOR && gmax <= 1e-4f) break;
@@ -1263,10 +1271,10 @@ static __device__ __noinline__ int solve_mixed64(double ubx, double uby, double 
     for (int k = 0; k < NM; ++k) {
       G[k] -= m[k];
       g32[k] = cvt_f32_rn(G[k]);
-      gmax = fmaxf(gmax, fabsf(g32[k]));
+      gmax = max_nan(gmax, fabsf(g32[k]));
     }
     if (gmax <= tolf) return NEWTON_OK;
-    // (a NaN residual fails the comparison)
+    // (a NaN residual fails both comparisons)
     if (n >= 6 || !(gmax < last)) return NEWTON_MAXIT;
     last = gmax;
     float h32[36];
@@ -1495,7 +1503,7 @@ __device__ __forceinline__ float exponent_bound(const float l[NM]) {
   const float dg = fmaf(4.0f, fabsf(l[3]) + fabsf(l[4]) + fabsf(l[5]),
                         fmaf(2.0f, fabsf(l[1]) + fabsf(l[2]),
                              mul_rn(16.0f, fabsf(l[6]) + fabsf(l[7]))));
-  return fabsf(1.0f + l[0]) + fmaxf(fmaxf(ax, ay), dg);
+  return fabsf(1.0f + l[0]) + max_nan(max_nan(ax, ay), dg);
 }
 
 // Refinement of the FP32 form in fixed point: as refine_fp64, lambda <- lambda +

@@ -453,7 +453,7 @@ __device__ __noinline__ bool prelude13(float ubx, float uby, float T, float l[M]
 #pragma unroll
     for (int k = 0; k < M; ++k) {
       g[k] = sum_of(mom, k) - m[k];
-      gmax = fmaxf(gmax, fabsf(g[k]));
+      gmax = max_nan(gmax, fabsf(g[k]));
     }
     *iters = it;
     if (!isfinite(gmax)) return false;
@@ -501,9 +501,10 @@ __device__ __noinline__ int solve13_mixed(double ubx, double uby, double T, doub
     for (int k = 0; k < M; ++k) {
       G[k] = sum_of(mom, k) - m[k];
       g32[k] = cvt_f32_rn(G[k]);
-      gmax = fmaxf(gmax, fabsf(g32[k]));
+      gmax = max_nan(gmax, fabsf(g32[k]));
     }
     if (gmax <= tolf) return OK;
+    // (a NaN residual fails both comparisons)
     if (n >= 6 || !(gmax < last)) return MAXIT;
     last = gmax;
     float L[M * (M + 1) / 2], d32[M], r32[M];
