@@ -95,7 +95,10 @@ typedef struct alb_handle alb_handle; /* opaque */
  *                (sensor_eps[2], sensor_alpha[1]), (10 sensor_eps[2],
  *                sensor_alpha[2]), constant beyond (sensor_eps increasing).
  *   newton_tol   stop when max_k |G_k| / rho <= newton_tol (paper: 1e-12).
- *   newton_maxit iteration cap.
+ *   newton_maxit cap on the iterations of a solve from one start. In the FP32 form
+ *                with 8 moments it is the cap of the FP64 Newton that takes
+ *                over where the FP32 Newton and its refinement fail (these
+ *                have caps of their own, 30 and 6).
  *   newton_start starting point of each equilibrium solve: ALB_START_AUTO
  *                (the node's multipliers of the previous step in the FP32
  *                form, the Maxwellian in FP64 plain), ALB_START_MAXWELLIAN,
@@ -115,8 +118,9 @@ typedef struct alb_handle alb_handle; /* opaque */
  *   moments      constraint set of the numerical equilibrium: 8 (Eqs.
  *                G0_8mom..G3yaa_8mom, the default) or 4 (the reduced model
  *                of App. C.2, Eq. feqNum_4Mom: mass, momentum and the energy
- *                trace; solved as the full set is in the FP32 form, by a 4x4
- *                Newton in FP64 in FP64 plain) on D2Q21; 13
+ *                trace; solved as the full set is in the FP32 form where
+ *                newton_maxit is at least 37, else by a 4x4 Newton in FP64) on
+ *                D2Q21; 13
  *                (Eqs. G0..G4yyaa: moments up to third order and the trace
  *                of the fourth, Eq. feqNum_13Mom with the x^3 monomial the
  *                printed exponent omits) on D2Q49.

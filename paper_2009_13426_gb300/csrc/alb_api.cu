@@ -197,11 +197,8 @@ int alb_create(const alb_config* cfg, alb_handle** out) {
   p.sensor = cfg->sensor;
   p.maxit = cfg->newton_maxit;
   p.warm = uses_previous_start(cfg) ? 1 : 0;
-  // An explicit Maxwellian start keeps the oracle's iteration (all steps in
-  // FP64), and so does a cap on the iterations that the mixed solve could
-  // exceed (30 FP32 steps and 7 FP64 residuals): what does not converge under it
-  // has to fail as before.
-  p.mixed64 = cfg->newton_start != ALB_START_MAXWELLIAN && cfg->newton_maxit >= 37 ? 1 : 0;
+  // An explicit Maxwellian start keeps the oracle's iteration, all steps in FP64.
+  p.mixed64 = cfg->newton_start != ALB_START_MAXWELLIAN && cfg->newton_maxit >= MIXED_MAXIT;
   p.overlap = cfg->shift_overlap;
   p.rule = cfg->shift_rule;
   p.moments = cfg->moments;

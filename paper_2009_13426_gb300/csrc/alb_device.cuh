@@ -54,6 +54,12 @@ __device__ __forceinline__ float to_p<float>(double v) { return cvt_f32_rn(v); }
 template <>
 __device__ __forceinline__ double to_p<double>(double v) { return v; }
 
+// Smallest cap on the iterations (Params::maxit) under which a solve may take its
+// early steps in FP32: from one start such a solve takes at most 30 FP32 steps and
+// 7 residuals in 64 bits (it may try two starts, as the FP64 iteration does, whose
+// cap is per start too). What does not converge under a smaller cap has to fail.
+constexpr int MIXED_MAXIT = 37;
+
 // Physical and numerical parameters of one flow, passed by value.
 struct Params {
   int nx, ny;

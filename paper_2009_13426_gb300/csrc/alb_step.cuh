@@ -86,9 +86,12 @@ static __device__ __noinline__ int solve_other(const Params& pr, const double* e
   for (int k = 0; k < NM; ++k) lam[k] = io->lam[k];
   io->fixed = false;
   if (pr.moments == 4) {
+    // (under a small cap on the iterations, the FP64 Newton alone)
     int it32 = 0, ev = 0, up = 0;
-    st = solve4_fix(ubx, uby, T, (float)pr.tol, warm, fixtab, reinterpret_cast<uint64_t*>(eq), B,
-                    lam, &it32, &ev, &up);
+    st = NEWTON_MAXIT;
+    if (pr.maxit >= MIXED_MAXIT)
+      st = solve4_fix(ubx, uby, T, (float)pr.tol, warm, fixtab, reinterpret_cast<uint64_t*>(eq), B,
+                      lam, &it32, &ev, &up);
     cnt.fp32_iters = it32;
     cnt.fp64_evals = ev;
     cnt.fp64_updates = up;
