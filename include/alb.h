@@ -353,7 +353,8 @@ typedef struct alb_batch alb_batch; /* opaque */
  *                  bounds the registers per thread).
  *   tile_w[3]      tile width in nodes for flows with nx < 128, with
  *                  nx < 512, and wider; the tile height is block / tile_w.
- *                  Powers of two in [8, block].
+ *                  Powers of two in [8, block]. Tiles of a flow with few
+ *                  rows are wider (no more than twice as high as the grid).
  *   dynamic        1: blocks fetch work items from an atomic counter;
  *                  0: block b takes items b, b + grid, b + 2 grid, ...
  *   blocks_per_sm  resident blocks per SM of the persistent grid (0: the

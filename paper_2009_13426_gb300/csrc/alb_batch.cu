@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "alb_batcher.h"
+#include "alb_tiles.h"
 
 using namespace alb;
 
@@ -128,6 +129,7 @@ cudaError_t GroupPlan::build_items(cudaStream_t s, int only_class) {
       const int tw = std::min(tuning_.tile_w[c], block);
       int lg = 0;
       while ((1 << lg) < tw) ++lg;
+      lg = tile_lg(lg, block, p.ny);
       const int th = block >> lg;
       for (int y0 = 0; y0 < p.ny; y0 += th)
         for (int x0 = 0; x0 < p.nx; x0 += (1 << lg)) items.push_back(WorkItem{(int)f, x0, y0, lg});

@@ -16,6 +16,7 @@
 #include <type_traits>
 
 #include "alb_step.cuh"
+#include "alb_tiles.h"
 
 namespace alb {
 
@@ -298,7 +299,7 @@ static dim3 grid_of(const Params& p) { return dim3((p.nx + BLOCK - 1) / BLOCK, p
 static dim3 step_grid(const Params& p, int block, int* lg) {
   int l = 3;
   while (l < 5 && (1 << l) < p.nx) ++l;
-  while ((1 << l) < block && (block >> l) >= 2 * p.ny) ++l;
+  l = tile_lg(l, block, p.ny);
   *lg = l;
   const int rows = block >> l;
   return dim3((p.nx + (1 << l) - 1) >> l, (p.ny + rows - 1) / rows);
