@@ -734,11 +734,16 @@ __device__ __forceinline__ void shift_multipliers(const R l[NM], R dx, R dy, R o
 // rounding, with two or three steps still to go. One FP32 step more would be
 // 20 % faster, but its rounding then shows in the last step: the tube parted
 // from the oracle by 1.1e-10 in 1000 steps where it stays below 1e-11 so.
-template <bool FACTOR>
+//
+// FRESH = true evaluates and factorises once more after the last step, so that
+// the factor is of the returned point: for the refinement in FP64, whose residuals
+// cost the most (2.4 a solve instead of 3.8 on random states; 200,000 solves of
+// alb_equilibrium 291 instead of 366 us).
+template <bool FACTOR, bool FRESH = false>
 __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int maxit, bool warm,
                                            float lam[NM], Fact32& fc, int* iters, float* gres,
                                            bool* stale) {
-  enum { START_WARM, START_MAXWELL, TRIAL, RETURNED };
+  enum { START_WARM, START_MAXWELL, TRIAL, RETURNED, FULL_STEP };
   *iters = 0;
   *stale = false;
   // Maxwellian multipliers with lambda_0 = 0 (fixed from the normalisation
@@ -821,7 +826,7 @@ __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int ma
     // FP32 exit at 1e-6, five times the FP32 residual's own noise (about
     // 2e-7): below that the FP32 steps only chase rounding, and the
     // refinement contracts by about 1e-4 per residual from either level
-    if (mode == RETURNED || gmax <= 1e-6f || it >= maxit) break;
+    if (mode == RETURNED || (FRESH && mode == FULL_STEP) || gmax <= 1e-6f || it >= maxit) break;
     solve32(fc, G, dl);
     gd = 0.0f;
 #pragma unroll
@@ -838,8 +843,13 @@ __device__ __forceinline__ int newton_fp32(float ubx, float uby, float T, int ma
       // by some 1e-3, so it still contracts by about that per residual, at
       // 0.6 more residuals a solve than with a fresh factor but without the
       // pass and the factorisation that one takes.
-      *stale = true;
+      // (FRESH takes them: the refinement in FP64 is the dearer part there.)
       ++it;
+      if (FRESH) {
+        mode = FULL_STEP;
+        continue;
+      }
+      *stale = true;
       break;
     }
     mode = TRIAL;
@@ -1783,6 +1793,16 @@ static __device__ __noinline__ int solve4_fix(double ubx, double uby, double T, 
   return NEWTON_OK;
 }
 
+// The FP32 phase of the refinement in FP64, with a fresh factor. A function of its
+// own: inlined beside the call of the refinement it spills (200,000 solves of
+// alb_equilibrium 291 us inlined, 257 us so).
+static __device__ __noinline__ int newton_fp32_fresh(float ubx, float uby, float T, bool warm,
+                                                     float lam[NM], Fact32& fc, int* iters,
+                                                     float* gres) {
+  bool stale;
+  return newton_fp32<true, true>(ubx, uby, T, 30, warm, lam, fc, iters, gres, &stale);
+}
+
 // Equilibrium of the FP32 form by FP32 Newton (from the warm start if given,
 // else from the Maxwellian; again from the Maxwellian if the warm start fails),
 // FP64 refinement, full FP64 Newton as the last fallback. The FP64 equilibrium
@@ -1807,8 +1827,7 @@ static __device__ __noinline__ int equilibrium_mixed(double ubx, double uby, dou
     for (int k = 0; k < NM; ++k) l32[k] = warm[k];
   for (;;) {
     int it32 = 0;
-    bool stale;
-    st = newton_fp32<true>(ubx32, uby32, T32, 30, w, l32, fc, &it32, &gres, &stale);
+    st = newton_fp32_fresh(ubx32, uby32, T32, w, l32, fc, &it32, &gres);
     cnt->fp32_iters += it32;
     if (st == NEWTON_OK || !w) break;
     w = false;
