@@ -477,15 +477,17 @@ __device__ __noinline__ bool prelude13(float ubx, float uby, float T, float l[M]
   }
 }
 
-// As newton13; *iters counts all steps. A status other than NEWTON_OK leaves the
-// solve to newton13.
+// As newton13; *iters32 and *iters count the steps in FP32 and in FP64. A status
+// other than NEWTON_OK leaves the solve to newton13.
 __device__ __noinline__ int solve13_mixed(double ubx, double uby, double T, double tol, double* eq,
-                                          const double* tab, double lam[M], int* iters) {
-  *iters = 0;
+                                          const double* tab, double lam[M], int* iters32,
+                                          int* iters) {
+  *iters32 = *iters = 0;
   if (!(T > 0.0) || !isfinite(T) || !isfinite(ubx) || !isfinite(uby)) return NEWTON_UNREALIZABLE;
   {
     float l32[M];
-    if (!prelude13(cvt_f32_rn(ubx), cvt_f32_rn(uby), cvt_f32_rn(T), l32, iters)) return SINGULAR;
+    if (!prelude13(cvt_f32_rn(ubx), cvt_f32_rn(uby), cvt_f32_rn(T), l32, iters32))
+      return SINGULAR;
 #pragma unroll
     for (int k = 0; k < M; ++k) lam[k] = cvt_f64(l32[k]);
   }
@@ -539,23 +541,29 @@ __device__ __noinline__ int solve13_mixed(double ubx, double uby, double T, doub
   }
 }
 
+struct Count {
+  unsigned iters = 0, iters32 = 0;  // Newton steps, those in FP32 among them
+  unsigned calls = 0, fail = 0, rec = 0, rec_fail = 0;
+};
+
 // The solve of the step and of the initial state: mixed precision, newton13
 // where that fails or is not asked for (Params::mixed64).
 __device__ __forceinline__ int solve13(const Params& pr, double ubx, double uby, double T,
-                                       double* eq, const double* tab, double lam[M], int* iters) {
+                                       double* eq, const double* tab, double lam[M], Count* cnt) {
   int st = SINGULAR;
-  if (pr.mixed64) st = solve13_mixed(ubx, uby, T, pr.tol, eq, tab, lam, iters);
+  if (pr.mixed64) {
+    int it32 = 0, it = 0;
+    st = solve13_mixed(ubx, uby, T, pr.tol, eq, tab, lam, &it32, &it);
+    cnt->iters32 += it32;
+    cnt->iters += it32 + it;
+  }
   if (st != OK && st != NEWTON_UNREALIZABLE) {
     int it = 0;
     st = newton13(ubx, uby, T, pr.tol, pr.maxit, eq, tab, lam, &it);
-    *iters = it;
+    cnt->iters += it;
   }
   return st;
 }
-
-struct Count {
-  unsigned iters = 0, calls = 0, fail = 0, rec = 0, rec_fail = 0;
-};
 
 // The sender of a rebuilt pull: its stored moments at the (possibly ghost)
 // position (sx, sy) and the central differences of u and T around it.
@@ -636,10 +644,8 @@ __device__ __forceinline__ void fallback_value(const Params& pr, const Sender& s
 __device__ __noinline__ int sender_solve(const Params pr, const Sender s, int Upx, int Upy,
                                          double* eq, const double* tab, double lam[M],
                                          Count* cnt) {
-  int it = 0;
-  const int st = s.rho > 0.0 ? solve13(pr, s.ux - Upx, s.uy - Upy, s.T, eq, tab, lam, &it)
+  const int st = s.rho > 0.0 ? solve13(pr, s.ux - Upx, s.uy - Upy, s.T, eq, tab, lam, cnt)
                              : NEWTON_UNREALIZABLE;
-  cnt->iters += it;
   cnt->calls += 1;
   return st;
 }
@@ -699,9 +705,7 @@ __device__ __forceinline__ void collide(const Params& pr, const double* col, dou
                                      select_shift_neighbours(uy, 1, nb, pr))
                           : lat_code(select_shift_kept(ux, Ux, pr), select_shift_kept(uy, Uy, pr));
   double lam[M];
-  int it = 0;
-  const int ns = rho > 0.0 ? solve13(pr, ubx, uby, T, eq, tab, lam, &it) : NEWTON_UNREALIZABLE;
-  cnt->iters += it;
+  const int ns = rho > 0.0 ? solve13(pr, ubx, uby, T, eq, tab, lam, cnt) : NEWTON_UNREALIZABLE;
   cnt->calls += 1;
   if (ns == NEWTON_OK) {
     const double gp = (2.0 * pr.cv - 2.0) * T;
@@ -756,6 +760,7 @@ __device__ __forceinline__ void collide(const Params& pr, const double* col, dou
 
 __device__ __forceinline__ void flush(unsigned long long* ctr, const Count& c) {
   warp_count(ctr + CTR_NEWTON_ITERS, c.iters);
+  warp_count(ctr + CTR_FP32_ITERS, c.iters32);
   warp_count(ctr + CTR_NEWTON_CALLS, c.calls);
   warp_count(ctr + CTR_NEWTON_FAIL, c.fail);
   warp_count(ctr + CTR_REC, c.rec);
@@ -946,8 +951,7 @@ __global__ void __launch_bounds__(B) init_kernel(InitArgs49 a) {
     const int code = lat_code(U0x, U0y);
     const bool ok = (r > 0.0) && (T > 0.0) && isfinite(r) && isfinite(T);
     double lam[M];
-    int it = 0;
-    const int ns = ok ? solve13(pr, ux - U0x, uy - U0y, T, eq, s_tab, lam, &it)
+    const int ns = ok ? solve13(pr, ux - U0x, uy - U0y, T, eq, s_tab, lam, &cnt)
                       : NEWTON_UNREALIZABLE;
     if (!ok) bad += 1;
     if (ok && ns != NEWTON_OK) cnt.fail += 1;
