@@ -106,11 +106,11 @@ typedef struct alb_handle alb_handle; /* opaque */
  *                sender's, multipliers of the previous step moved to the
  *                lattice of the solve; 8 more planes per buffer). The root is
  *                unique, so the start changes only the path and round-off;
- *                ALB_START_MAXWELLIAN follows the oracle's iteration with
- *                every step in FP64. The other starts of FP64 plain take the
- *                iteration's early steps in FP32 (where newton_maxit is at
- *                least 37) and the last ones, from a residual of about 1e-3
- *                on, in FP64.
+ *                ALB_START_MAXWELLIAN follows the oracle's iteration, in FP64
+ *                plain and on D2Q49 with every step in FP64. The other
+ *                starts take the iteration's early steps there in FP32
+ *                (where newton_maxit is at least 37) and the last ones, from
+ *                a residual of about 1e-3 on, in FP64.
  *   shift_overlap w in [0, 1]: each shift's range widened by w on both
  *                sides, U - n0 - w < u <= U + 1 - n0 + w, so that the ranges
  *                of neighbouring shifts overlap (Sec. III.A.2); 0 (the
@@ -166,18 +166,19 @@ typedef struct {
   uint64_t steps;
   uint64_t node_updates;
   uint64_t newton_iterations;       /* Newton steps of FP64 solves, node and rebuild
-                                       equilibria (FP64 plain: all steps, those in
-                                       fp32_iterations included) */
+                                       equilibria (FP64 plain and D2Q49: all steps,
+                                       those in fp32_iterations included) */
   uint64_t newton_failures;         /* node equilibria that failed */
   uint64_t reconstructions;         /* missing pulls rebuilt (Grad) */
   uint64_t reconstruction_failures; /* rebuilds that fell back */
   uint64_t newton_calls;            /* equilibrium solves, node and rebuild */
-  uint64_t fp64_evaluations;        /* FP64 evaluations of the 21 exponentials */
+  uint64_t fp64_evaluations;        /* residuals that evaluate the 21 exponentials, in
+                                       FP64 or (FP32 form) in 64-bit fixed point; not
+                                       counted on D2Q49 */
   uint64_t fp32_iterations;         /* Newton steps in FP32 */
-  uint64_t fp64_updates;            /* FP32 form: residual evaluations that updated
-                                       the 21 FP64 populations multiplicatively
-                                       after a small step instead of evaluating
-                                       the exponentials (not in fp64_evaluations) */
+  uint64_t fp64_updates;            /* FP32 form: residuals that update the 21
+                                       populations multiplicatively after a small
+                                       step instead (not in fp64_evaluations) */
 } alb_stats;
 
 /* Fill *cfg with defaults: 64x64, D2Q21, u_max 2, nu 1e-3, gamma 1.4,
@@ -289,10 +290,13 @@ const char* alb_last_error(void);
 /* Numerical equilibrium (Eqs. exponential, feqNum_8Mom, constraints
  * G0_8mom..G3yaa_8mom) of n states given in the lattice frame: rho[k],
  * relative velocity (ubx[k], uby[k]) and T[k]; stop at max|G|/rho <= tol.
- * precision selects the solver of the step kernels: ALB_FP64_PLAIN, damped
- * Newton in FP64; ALB_FP32_FORM, Newton in FP32 refined with FP64 residuals
- * (full FP64 Newton if that fails). Writes feq[k*21 + i] (velocity order of
- * alb_velocities), lambda[k*8 + j] if lambda != NULL (order 0, x, y, xx, xy,
+ * precision: ALB_FP64_PLAIN, damped Newton with every step in FP64;
+ * ALB_FP32_FORM, Newton in FP32 refined with FP64 residuals (full FP64 Newton
+ * if that fails), which gives FP64 multipliers. Steps and initial states run
+ * these where their own solvers (residuals in fixed point, early steps in
+ * FP32) do not reach or are not asked for; the root is the same. Writes
+ * feq[k*21 + i] (velocity order of alb_velocities), lambda[k*8 + j] if
+ * lambda != NULL (order 0, x, y, xx, xy,
  * yy, x|xi|^2, y|xi|^2), iters[k] (FP64 Newton steps, or FP64 residual
  * evaluations, full and multiplicative, for ALB_FP32_FORM; the latter's
  * populations are exponential-family members to about 1e-10 relative, their
@@ -374,7 +378,8 @@ int alb_batch_variants(int precision, int* count, int* block, int* min_blocks);
  * parameters and precisions; each cfg's stream is ignored). All work runs on
  * `stream` (cudaStream_t; NULL: the batch creates one; not the legacy
  * default stream, which cannot be captured). Default launch shape: variant
- * 0, tiles of 64 / 128 / 128 nodes (at most the block), dynamic items. */
+ * 4 (256 threads) in the FP32 form, 0 in FP64 plain, tiles 32 nodes wide,
+ * dynamic items. */
 int alb_batch_create(const alb_config* cfgs, int nflows, void* stream, alb_batch** out);
 
 /* Handle of flow i (0 <= i < nflows), owned by the batch: use it with
