@@ -60,10 +60,10 @@ from paper_2009_13426_gb300 import costmodel, flows  # noqa: E402
 METRIC = "adaptive D2Q21 MLUPS, FP32 form vs FP64 plain at stated error; serve p50/p99"
 # DRAM bytes (read + write) per node update of step_kernel<float>, from one
 # ncu capture of the 2048^2 case of the same flow (dram__bytes_read.sum +
-# dram__bytes_write.sum = 876.8 + 1117.8 MB per launch for 4,194,304 nodes,
+# dram__bytes_write.sum = 876.1 + 1107.4 MB per launch for 4,194,304 nodes,
 # first steps, kinetic sensor on); the traffic grows in proportion to the
 # nodes, so a 4096^2 launch moves 16,777,216 x this.
-TRAFFIC_BYTES_PER_NODE_FP32 = 475.6
+TRAFFIC_BYTES_PER_NODE_FP32 = 472.9
 UNIT = "MLUPS"
 NU = 1e-5
 # The kinetic sensor (Sec. IV.A.2) is on in every timed flow: without it the
@@ -764,9 +764,14 @@ def run_ours(args, world, rank, local):
                "steps": k49, "ms_per_step": round(ms49 / k49, 3),
                "kernel": "q49::step_kernel",
                "per_node": {k: round(d49[k] / (N49 * k49), 4)
-                            for k in ("newton_iterations", "newton_calls", "reconstructions")},
+                            for k in ("newton_iterations", "fp32_iterations", "newton_calls",
+                                      "reconstructions")},
                "failures": {"node": d49["newton_failures"],
                             "rebuild": d49["reconstruction_failures"]}}
+        t49 = 2.0 * costmodel.q49_slots(d49, N49 * k49) / (ms49 * 1e-3) / 1e12
+        q49["roofline"] = {"bound": "alu", "achieved": round(t49, 4),
+                           "peak": round(costmodel.FP64_PEAK_TFLOPS, 4), "unit": "TFLOP/s",
+                           "frac": round(t49 / costmodel.FP64_PEAK_TFLOPS, 4)}
         fl.close()
 
     e2e = None

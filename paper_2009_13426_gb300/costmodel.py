@@ -3,9 +3,10 @@
 FP64 plain and D2Q49 are bound by the FP64 pipe, not by HBM: on GB300 the FP64
 rate is 1/62 of the FP32 rate. The FP32 form forms its residuals in fixed point
 on the integer pipe and is bound by instruction issue and the latency of its
-chains at 8 to 16 warps per SM (issue_instr below); the FP32-form counts of
-fp64_slots describe its FP64 refinement, which now serves only states outside
-the fixed-point range.
+chains at 8 to 16 warps per SM. issue_instr, plain_slots and q49_slots count the
+work of the step kernels; fp64_slots and method_floor count solves whose
+residuals (FP32 form) or Newton steps (FP64 plain) are all in FP64, as those of
+alb_equilibrium are.
 
 FP64 arithmetic is counted in issue slots: one
 slot per FP64 lane operation (DFMA, DADD, DMUL, DMNMX, DSETP, hardware
@@ -186,7 +187,7 @@ def issue_instr(stats: dict) -> float:
     after each phase (2048^2 and 1024^2 shear layers): pulls, moments, collision
     and store 3,300 per node, 650 per FP32 evaluation pass with its factorisation,
     1,150 per fixed-point evaluation or update, 2,000 per rebuilt pull. It gives
-    6,830 per node where ncu counts 6,858 (2048^2, first steps)."""
+    6,742 per node where ncu counts 6,737 (2048^2, second launch)."""
     return (3300.0 * stats["node_updates"]
             + 650.0 * (stats["fp32_iterations"] + stats["newton_calls"])
             + 1150.0 * (stats["fp64_evaluations"] + stats.get("fp64_updates", 0))
@@ -205,9 +206,9 @@ def plain_slots(stats: dict) -> float:
     return PLAIN_MIXED_CALIBRATION * raw
 
 
-# ncu counted 2,156 FP64-pipe thread instructions per node on the 1024^2 layer (4.20
-# evaluations, 3.13 FP64 steps, 1.08 solves, 0.20 rebuilt pulls per node).
-PLAIN_MIXED_CALIBRATION = 2156.0 / 1980.7
+# ncu counted 2,135 FP64-pipe thread instructions per node on the 1024^2 layer (4.18
+# evaluations, 3.11 FP64 steps, 1.07 solves, 0.19 rebuilt pulls per node).
+PLAIN_MIXED_CALIBRATION = 2134.7 / 1972.6
 
 
 def method_floor(mlups: float) -> dict:
@@ -244,29 +245,28 @@ if __name__ == "__main__":
 
 # ---------------------------------------------------------------- D2Q49
 
-# Slots of the D2Q49 step (alb_q49.cu), counted like the rest of this file:
-# per Newton step, moments from the row sums (664), residual and its maximum
-# (45), Jacobian entries from the moments (140), Cholesky with reciprocal
-# pivots (690), two triangular solves (182), one line-search evaluation of
-# the 49 exponentials with the dual value (1060); per solve, targets, the
-# Maxwellian start's evaluation, log and normalisation (1220); per node,
-# moments, shift choice and BGK store (550); per rebuilt pull, the sender's
-# central differences, its exponential from the shared solve's multipliers
-# and the Grad factors (107).
-Q49_PER_ITER = 664 + 45 + 140 + 690 + 182 + 13 + 1060
-Q49_PER_CALL = 1220
+# Slots of the D2Q49 step (alb_q49.cu) whose early Newton steps run in FP32: per
+# evaluation in FP64 (one more than the steps in FP64 of a solve) the exponents and
+# the 45 moments of the tensor-product pass (610), 49 exponentials (7 each), the
+# targets and the residual (53); per step in FP64 the Jacobian's entries from the
+# moments (48) with their products by the step (169), and the multipliers' update
+# (26); per node moments, shift choice and BGK store (550); per rebuilt pull the
+# sender's central differences, its exponential from the shared solve's
+# multipliers and Grad's factors (412, from two captures at different shares of
+# rebuilt pulls: the divisions weigh most).
+Q49_PER_EVAL = 610 + 49 * 7 + 53
+Q49_PER_STEP = 48 + 169 + 26
 Q49_PER_NODE = 550
-Q49_PER_REBUILD = 12 + 9 + 9 + 1 + 40 + 3 * W_DIV + 8
-# ncu counted 30,696 FP64-pipe thread instructions per node on the 512^2
-# shear layer (7.10 Newton steps, 1.26 solves, 1.32 rebuilt pulls per node),
-# where the count above gives 22,067.
-CALIBRATION["q49"] = 30696.0 / 22067.0
+Q49_PER_REBUILD = 412
+# ncu counted 8,577 FP64-pipe thread instructions per node on the 512^2 shear
+# layer (3.39 FP64 steps, 1.18 solves, 1.31 rebuilt pulls per node), where the
+# count above gives 6,513.
+CALIBRATION["q49"] = 8577.0 / 6513.0
 
 
 def q49_slots(delta, node_updates):
-    """FP64 slots of D2Q49 launches with every Newton step in FP64 (an explicit
-    Maxwellian start), from their counters."""
-    rebuilds = delta["reconstructions"]
-    raw = (Q49_PER_ITER * delta["newton_iterations"] + Q49_PER_CALL * delta["newton_calls"]
-           + Q49_PER_NODE * node_updates + Q49_PER_REBUILD * rebuilds)
+    """FP64 slots of D2Q49 launches, from their counters."""
+    steps = max(0, delta["newton_iterations"] - delta["fp32_iterations"])
+    raw = (Q49_PER_EVAL * (steps + delta["newton_calls"]) + Q49_PER_STEP * steps
+           + Q49_PER_NODE * node_updates + Q49_PER_REBUILD * delta["reconstructions"])
     return CALIBRATION["q49"] * raw
