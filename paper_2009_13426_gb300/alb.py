@@ -419,6 +419,8 @@ def alb_batch_get_tuning(b, precision) -> dict:
 
 def alb_batch_set_tuning(b, precision, variant=0, tile_w=(64, 128, 128), dynamic=1,
                          blocks_per_sm=0):
+    """Sets the whole launch shape (the defaults here are not the batch's own, which
+    are variant 4 in the FP32 form, 0 in FP64 plain, and tiles 32 nodes wide)."""
     t = alb_batch_tuning(variant, (ctypes.c_int * 3)(*tile_w), dynamic, blocks_per_sm)
     return _check(lib().alb_batch_set_tuning(b, int(precision), ctypes.byref(t)))
 

@@ -179,9 +179,10 @@ cudaError_t GroupPlan::flip(cudaStream_t s) const { return launch_flip(d_cur_, n
     if (e_ != cudaSuccess) return cuda_error(e_, what);     \
   } while (0)
 
-// Default launch shape of a precision: 256 threads without spills in the FP32 form
-// (variant 4; see launch_step for the shapes by size), variant 0 in FP64 plain;
-// tiles 32 nodes wide.
+// Default launch shape of a precision: 256 threads, one block per SM, in the FP32
+// form (variant 4, the fewest spills of its variants: 140 bytes a thread stored
+// against 288 and more; launch_step has the shapes by size of a single flow),
+// variant 0 in FP64 plain; tiles 32 nodes wide.
 Tuning default_tuning(int precision) {
   Tuning t;
   if (precision == ALB_FP32_FORM) t.variant = 4;

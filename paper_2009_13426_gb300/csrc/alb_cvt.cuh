@@ -1,8 +1,9 @@
 // Conversions to and from FP64 on the integer pipe.
 //
-// On GB300 the FP64 pipe (2 operations per clock and SM) bounds the FP32
-// form's step, and it also executes every conversion to or from FP64. The
-// conversions of the step's hot loops are therefore assembled from the IEEE
+// The FP64 pipe of GB300 (2 operations per clock and SM) also executes every
+// conversion to or from FP64. It bounds FP64 plain and D2Q49, and it bounded the
+// FP32 form before its residuals moved to fixed point. The conversions of the
+// steps' hot loops are therefore assembled from the IEEE
 // 754 binary64 / binary32 bit fields with integer operations, which issue at
 // the integer pipe's rate beside the FP64 work:
 //   binary64: sign (1) | exponent (11, bias 1023) | fraction (52)

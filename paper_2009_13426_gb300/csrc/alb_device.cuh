@@ -84,8 +84,8 @@ struct Params {
   double wlo[7], whi[7];  // widened range of shift n = j - 3: ((n - n0) - w, ((n + 1) - n0) + w]
 };
 
-// Comparisons of the criterion on the integer pipe: the FP64 pipe bounds the
-// step, and an FP64 compare takes one of its slots. order_key maps a double's
+// Comparisons of the criterion on the integer pipe: an FP64 compare takes a slot
+// of the FP64 pipe, which bounds FP64 plain. order_key maps a double's
 // bits to a signed integer in IEEE order (negative values have their
 // magnitude bits flipped). Integer order then equals IEEE order for all
 // non-NaN values except +0 against -0, which cannot meet here: the host's

@@ -347,12 +347,16 @@ static cudaError_t launch_step_shape(const FlowDev& f, cudaStream_t s) {
 // 512^2 shear 1.44 / 1.46, but 700^2 2.53 / 2.46 and 1400^2 vortex 7.73 / 7.39).
 //
 // FP32 form, ms a step with 256 threads and 255 registers (one block per SM),
-// 384 and 168, and two blocks of 256 and 128, which spill but keep 16 warps:
-//   64^2 vortex 0.103 / 0.149 / 0.127    201^2 Riemann 0.105 / 0.121 / 0.131
-//   512^2 shear 0.260 / 0.277 / 0.283    700^2 shear 0.376 / 0.368 / 0.419
-//   1021 x 733 shear 0.567 / 0.545 / 0.580   1400^2 vortex 1.01 / 0.97 / 0.90
-//   4096^2 shear 9.94 / 9.68 / 10.0
-// Few tiles want the shortest chain through one block, many the most warps.
+// 384 and 168, and two blocks of 256 and 128, which spill most but keep 16 warps:
+//   600^2 shear 0.288 / 0.296 / -        600^2 vortex 0.209 / 0.203 / -
+//   800^2 shear 0.441 / 0.423 / -        800^2 Riemann 0.476 / 0.455 / -
+//   1030^2 shear 0.674 / 0.643 / 0.613   1030^2 vortex 0.557 / 0.530 / 0.483
+//   1400^2 shear 1.08 / 1.01 / 0.93      1400^2 Riemann 1.11 / 1.05 / 1.02
+//   2048^2 shear 2.05 / 1.93 / 1.70      2900^2 Riemann 4.15 / 3.96 / 3.75
+//   4096^2 shear 7.44 / 7.02 / 6.04
+// and below, in an earlier build, 64^2 vortex 0.103 / 0.149 / 0.127, 201^2 Riemann
+// 0.105 / 0.121 / 0.131, 512^2 shear 0.260 / 0.277 / 0.283, 700^2 shear 0.376 / 0.368
+// / 0.419. Few tiles want the shortest chain through one block, many the most warps.
 // Blocks smaller than 256 lose threads for an interface tile's rebuild solves
 // (201^2: 0.161 with 128, 0.207 with 64 where 256 took 0.151). Grids of fewer
 // than 8 rows do not fill the 32 x 8 tile: 128 threads (2048 x 4 tube 0.048 ms).

@@ -161,9 +161,9 @@ __device__ __forceinline__ double exp_scaled(double q, int n, const double* tab)
 // to -s N / ln2, r = -s - n ln2/N in two parts, exp(r) by its degree-4 Taylor
 // polynomial, times 2^(n/N) = 2^(n >> 8) tab[n & 255].
 // n comes from an FP32 copy of s: within |s| <= 745 (past which the result is 0
-// or +inf anyway) FP32 holds s N / ln2 to 0.02, so n is the nearest integer or
-// its neighbour near a tie, |r| <= 0.52 ln2/256, and the polynomial's remainder
-// stays below 5e-17. The copy, n and its way back run on the integer pipe: 7 FP64
+// or +inf anyway) FP32 holds s N / ln2 to 0.031, so n is the nearest integer or
+// its neighbour near a tie, |r| <= 0.531 ln2/256, and the polynomial's remainder
+// stays below 5.2e-17. The copy, n and its way back run on the integer pipe: 7 FP64
 // operations (9 with the index rounded in FP64). Past |s| of 5.8e6 the
 // float-to-int rounding saturates and the limits hold; a NaN gives n = 0 and
 // passes through the polynomial.
@@ -189,9 +189,9 @@ __device__ __forceinline__ double exp_neg(double s, const double* tab) {
 // updates leave, both far below the FP32 storage of the populations.
 // The table index n nearest to -s N / ln2 comes from s32, an FP32 value of
 // the same exponent: within |s| <= 745 (past which the result is 0 or +inf
-// anyway) FP32 holds s to 5e-5, a fiftieth of ln2/N, so n is the nearest
-// integer or its neighbour at a tie and |r| stays below 0.52 ln2/N
-// (truncation r^3/3! below 4.7e-10). 4 FP64 operations: the reduction, the
+// anyway) FP32 holds s N / ln2 to 0.031, so n is the nearest integer or its
+// neighbour near a tie and |r| stays below 0.531 ln2/N (truncation r^3/3! below
+// 5e-10). 4 FP64 operations: the reduction, the
 // polynomial and the scaling (n reaches FP64 exactly on the integer pipe).
 // For |s32 N / ln2| >= 2^31 the float-to-int rounding saturates and e takes
 // the limits; a NaN gives n = 0 and passes through the polynomial.

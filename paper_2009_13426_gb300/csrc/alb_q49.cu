@@ -2,7 +2,8 @@
 // Sec. IV.B): the same adaptive step - pull in the receiver's lattice, Grad
 // rebuild of missing pulls, moments, next lattice, numerical equilibrium, BGK
 // (or the App. E collision) - on the D2Q49 lattice {-3..3}^2 with the
-// 13-moment equilibrium of Eqs. G0..G4yyaa / feqNum_13Mom. FP64 throughout.
+// 13-moment equilibrium of Eqs. G0..G4yyaa / feqNum_13Mom. FP64 throughout, but
+// for the early Newton steps of a solve.
 //
 // Velocity i = (x, y) has index i = (x + 3) + 7 (y + 3). One thread per node;
 // a block is a tile of 8 x 8 nodes. Each thread owns two columns of the

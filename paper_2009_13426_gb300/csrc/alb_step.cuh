@@ -64,7 +64,9 @@ struct SolveIO {
   bool warm, fixed;
 };
 
-// Counts of a solve, added to the flow's counters by the lanes that made one.
+// Counts of a solve, added to the flow's counters by the lanes that made one. Which
+// lanes of the warp run this together does not matter: each of them goes on to the
+// sum with the mask that names them, and every lane's count is in one such sum.
 __device__ __forceinline__ void lanes_count(unsigned long long* ctr, unsigned v) {
   const unsigned m = __activemask();
   const unsigned sum = __reduce_add_sync(m, v);
